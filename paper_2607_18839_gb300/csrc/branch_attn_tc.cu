@@ -56,6 +56,13 @@
 //               the next unit's metadata before the epilogue.
 // One split: the unit writes the final bf16 output and lse.  Several splits:
 // it writes its normalised fp32 partial and lse for merge.cu.
+// Code size: every CTA fetches the kernel's instructions anew, at some 150
+// cycles a 128-byte line on a cold path, and the roles' hot loops share one
+// instruction cache.  Code off the softmax's inner loop therefore exists
+// once and keeps its loops (producers, page look-ups), and divides by
+// multiplying: 124 KB of instructions became 64 KB, which took one call of
+// c3's shape from 41.4 to 37.6 us, of a scattered paged batch from 75.8 to
+// 68.3 us, and the attention of c5's shape from 133.3 to 129.7 us.
 // All waits are bounded; a timeout sets HPD_DEVERR_TIMEOUT, every role
 // leaves its loop, and the CTA drains its in-flight copies and MMAs, frees
 // its TMEM and exits.  No role waits on a hardware barrier (bar.sync) inside
@@ -111,6 +118,7 @@ struct TcLayout {
   static constexpr uint32_t kChunkBytes = kRows * 128;  // 128 rows x 128 bytes
   static constexpr uint32_t kTileBytes = kChunks * kChunkBytes;
   static constexpr int kKStages = 3, kVStages = 3;
+  static_assert(kKStages == kVStages, "one producer code for both rings");
   static constexpr uint32_t kK = 0;
   static constexpr uint32_t kV = kK + kKStages * kTileBytes;
   static constexpr uint32_t kMeta = kV + kVStages * kTileBytes;  // 2 UnitMeta slots
@@ -254,11 +262,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         u = __shfl_sync(0xffffffffu, u, 0);
         if (u >= p.n_units || aborted(sh)) break;
         if (p.unit_order) u = p.unit_order[u];  // longest units first
-        const int split = u % p.S_p;
-        const int g = (u / p.S_p) % p.H_kv;
-        const int tile = u / (p.S_p * p.H_kv);
+        const int us = p.div_S(u), split = u - us * p.S_p;
+        const int tile = p.div_Hkv(us), g = us - tile * p.H_kv;
         // the page owning the tile: page d has ceil(#branches(d) * m / TT) tiles
         int d = -1, lt = 0, b0 = 0, b1 = 0;
+#pragma unroll 1
         for (int d0 = 0, base = 0; d0 < p.n_docs && base <= tile; d0 += 32) {
           const int dd = d0 + lane;
           int tiles = 0, c0 = 0, c1 = 0;
@@ -269,10 +277,10 @@ __global__ void __launch_bounds__(kThreads, 1)
               flag_error(p.err, HPD_DEVERR_BRANCH_CU);
               c1 = c0;
             }
-            tiles = ceil_div_i((c1 - c0) * m, TT);
+            tiles = p.div_tile((c1 - c0) * m + TT - 1);
           }
           int incl = tiles;
-#pragma unroll
+#pragma unroll 1
           for (int o = 1; o < 32; o <<= 1) {
             const int v = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += v;
@@ -297,10 +305,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0 && bad_prefix) flag_error(p.err, HPD_DEVERR_PREFIX_CU);
         const int tok0 = b0 * m + lt * TT;
         const int ntok = min(TT, (b1 - b0) * m - lt * TT);
-        const int b_lo = tok0 / m;
-        const int nbc = (tok0 + ntok - 1) / m - b_lo + 1;
+        const int b_lo = p.div_m(tok0);
+        const int nbc = p.div_m(tok0 + ntok - 1) - b_lo + 1;
         // private lengths, packed page offsets and fork limits of the branches
         int base = 0, kmax = 0;
+#pragma unroll 1
         for (int c0 = 0; c0 < nbc; c0 += 32) {
           const int bl = c0 + lane;
           int np = 0;
@@ -325,7 +334,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             np = ceil_div_i(Lb, kPage);
           }
           int incl = np;
-#pragma unroll
+#pragma unroll 1
           for (int o = 1; o < 32; o <<= 1) {
             const int v = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += v;
@@ -333,51 +342,44 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (bl < nbc) M.page_start[bl] = base + incl - np;
           base += __shfl_sync(0xffffffffu, incl, 31);
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
+        kmax = __reduce_max_sync(0xffffffffu, kmax);
         const int P_s = base;
         if (lane == 0) M.page_start[nbc] = P_s;
         __syncwarp();
-        // packed suffix page ids (valid ids only), four lookups in flight
+        // packed suffix page ids: every lookup in flight, then the valid ones kept
         const int n_tab = min(P_s, kPageCap);
-        for (int gp0 = 0; gp0 < n_tab; gp0 += 128) {
-          int addr[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int gp = gp0 + q * 32 + lane;
-            addr[q] = -1;
-            if (gp < n_tab) {
-              int lo = 0, hi = nbc;  // largest bl with page_start[bl] <= gp
-              while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (M.page_start[mid] <= gp) lo = mid; else hi = mid;
-              }
-              addr[q] = (b_lo + lo) * p.max_pages + (gp - M.page_start[lo]);
-            }
+#pragma unroll 1
+        for (int gp = lane; gp < n_tab; gp += 32) {
+          int lo = 0, hi = nbc;  // largest bl with page_start[bl] <= gp
+          while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (M.page_start[mid] <= gp) lo = mid; else hi = mid;
           }
-          int pg[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) pg[q] = addr[q] >= 0 ? p.page_table[addr[q]] : 0;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            if (addr[q] < 0) continue;
-            if (pg[q] < 0 || pg[q] >= p.num_pages) {
-              flag_error(p.err, HPD_DEVERR_PAGE_ID);
-              pg[q] = 0;
-            }
-            M.page_tab[gp0 + q * 32 + lane] = pg[q];
-          }
+          cp_async4(smem_u32(&M.page_tab[gp]),
+                    p.page_table + static_cast<size_t>(b_lo + lo) * p.max_pages +
+                        (gp - M.page_start[lo]));
         }
+        cp_async_commit();
+        cp_async_wait<0>();
+#pragma unroll 1
+        for (int gp = lane; gp < n_tab; gp += 32)
+          if (static_cast<unsigned>(M.page_tab[gp]) >= static_cast<unsigned>(p.num_pages)) {
+            flag_error(p.err, HPD_DEVERR_PAGE_ID);
+            M.page_tab[gp] = 0;
+          }
         const int N = ceil_div_i(kmax, kBlk) + ceil_div_i(P_s, kPagesPerBlock);
-        const int blk_lo = static_cast<int>(static_cast<long long>(split) * N / p.S_p);
-        const int blk_hi = static_cast<int>(static_cast<long long>(split + 1) * N / p.S_p);
+        // (a unit has fewer than 2^27 blocks and at most 8 splits)
+        const int blk_lo = p.div_S(split * N), blk_hi = p.div_S((split + 1) * N);
         const int nrows = ntok * G;
         if (blk_hi <= blk_lo) {
           // no key in this split: zero output (one split) or an empty partial
+#pragma unroll 1
           for (int r = lane; r < nrows; r += 32) {
-            const size_t pair = static_cast<size_t>(tok0 + r / G) * p.H_q + g * G + r % G;
+            const int rt = p.div_G(r);
+            const size_t pair = static_cast<size_t>(tok0 + rt) * p.H_q + g * G + r - rt * G;
             if (p.S_p == 1) {
               uint4 *o = reinterpret_cast<uint4 *>(p.out + pair * D);
+#pragma unroll 1
               for (int c = 0; c < D / 8; ++c) o[c] = make_uint4(0u, 0u, 0u, 0u);
               if (p.lse) p.lse[pair] = NEG_INF;
             } else {
@@ -426,7 +428,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       prefetch_tmap(&tm_v8);
     }
     __syncwarp();
-    int jbase = 0, issued_k = 0, issued_v = 0;
+    // (one copy of this code, loops left as loops: a CTA of a small step runs
+    // it once or twice, and is bound by fetching its instructions)
+    uint64_t *const full = is_k ? sh.k_full : sh.v_full, *const empty = is_k ? sh.k_empty : sh.v_empty;
+    const CUtensorMap *const prefix_map = is_k ? &tm_k : &tm_v;
+    const CUtensorMap *const page_map = is_k ? &tm_kc : &tm_vc;
+    const CUtensorMap *const run_map = is_k ? &tm_k8 : &tm_v8;
+    const uint32_t ring = sbase + (is_k ? L::kK : L::kV);
+    const bool paged_prefix = p.prefix_page_table != nullptr;
+    int issued = 0;  // ring entries
     bool ok = true;
     for (int k = 0; ok; ++k) {
       const int slot = k & 1;
@@ -435,105 +445,74 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!M.valid) break;
       const int g = M.g, nP = M.nP, pc0 = M.pc0, blk_lo = M.blk_lo, nb = M.n_blocks;
       const int P_s = M.page_start[M.nbc];
-      // page id of packed suffix page gp (past the shared-memory table: looked
-      // up again; an id out of range was flagged by the scheduler)
-      auto page_of = [&](int gp) -> int {
-        if (gp < kPageCap) return M.page_tab[gp];
-        int lo = 0, hi = M.nbc;
-        while (hi - lo > 1) {
-          const int mid = (lo + hi) >> 1;
-          if (M.page_start[mid] <= gp) lo = mid; else hi = mid;
+      // entry -1 of the K ring: the unit's Q tile, tokens [tok0, tok0 + TT),
+      // heads of KV head g
+#pragma unroll 1
+      for (int j = is_k ? -1 : 0; j < nb; ++j) {
+        const int jb = blk_lo + j;
+        const bool contiguous = j < 0 || (jb < nP && !paged_prefix);
+        // A paged block is 8 pages (lane i < 8 holds page i, looked up before
+        // waiting for the ring slot); pages past the last one any row sees
+        // repeat it (finite values, never visible).
+        int pg = 0;
+        if (!contiguous && lane < kPagesPerBlock) {
+          if (jb < nP) {
+            pg = prefix_page(p, M.doc, min(jb * kPagesPerBlock + lane, M.pp_last));
+          } else {
+            const int gp = min((jb - nP) * kPagesPerBlock + lane, P_s - 1);
+            if (gp < kPageCap) {
+              pg = M.page_tab[gp];
+            } else {  // past the shared-memory table: looked up again
+              int lo = 0, hi = M.nbc;
+              while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (M.page_start[mid] <= gp) lo = mid; else hi = mid;
+              }
+              pg = p.page_table[static_cast<size_t>(M.b_lo + lo) * p.max_pages +
+                                (gp - M.page_start[lo])];
+              if (pg < 0 || pg >= p.num_pages) {
+                flag_error(p.err, HPD_DEVERR_PAGE_ID);
+                pg = 0;
+              }
+            }
+          }
         }
-        const int pg = p.page_table[static_cast<size_t>(M.b_lo + lo) * p.max_pages +
-                                    (gp - M.page_start[lo])];
-        if (pg < 0 || pg >= p.num_pages) {
-          flag_error(p.err, HPD_DEVERR_PAGE_ID);
-          return 0;
-        }
-        return pg;
-      };
-      // paged prefix: lane i < 8 fetches the pool page of prefix page
-      // 8 jb + i (pages past the last one any row sees repeat it: finite
-      // values, never visible); called before waiting for the ring slot so
-      // the lookup overlaps the wait
-      const bool paged_prefix = p.prefix_page_table != nullptr;
-      auto prefix_pid = [&](int jb) -> int {
-        if (!paged_prefix || jb >= nP || lane >= kPagesPerBlock) return 0;
-        return prefix_page(p, M.doc, min(jb * kPagesPerBlock + lane, M.pp_last));
-      };
-      // one block of K (or V) into stage `dst`.  A paged block is 8 pages
-      // (lane i < 8 holds page i); when they are consecutive pool pages one
-      // 8-page box loads them all, else one box per page.
-      auto load_block = [&](int jb, int pid, uint32_t dst, uint32_t b,
-                            const CUtensorMap *prefix_map, const CUtensorMap *page_map,
-                            const CUtensorMap *run_map) {
-        mbar_arrive_expect_tx_elect(b, L::kTileBytes);
-        if (jb < nP && !paged_prefix) {
+        const int e = issued, s = e % L::kKStages;
+        if (e >= L::kKStages && !(ok = wait_bar(empty[s], ((e / L::kKStages) - 1) & 1))) break;
+        ++issued;
+        const uint32_t dst = ring + s * L::kTileBytes, b = bar(full[s]);
+        mbar_arrive_expect_tx_elect(b, j < 0 ? L::kChunks * TT * G * 128 : L::kTileBytes);
+        if (contiguous) {
+#pragma unroll 1
           for (int c = 0; c < L::kChunks; ++c)
-            tma_load_3d_elect(dst + c * L::kChunkBytes, prefix_map, b, c * 64, g, pc0 + jb * kBlk);
-          return;
+            tma_load_3d_elect(dst + c * L::kChunkBytes, j < 0 ? &tm_q : prefix_map, b, c * 64,
+                              j < 0 ? g * G : g, j < 0 ? M.tok0 : pc0 + jb * kBlk);
+          continue;
         }
-        int pg = pid;
-        if (jb >= nP && lane < kPagesPerBlock)  // slots past the last page repeat it
-          pg = page_of(min((jb - nP) * kPagesPerBlock + lane, P_s - 1));
+        // consecutive pool pages load as one 8-page box, else one box per page
         const int next = __shfl_down_sync(0xffffffffu, pg, 1);
         const unsigned run =
             __ballot_sync(0xffffffffu, lane < kPagesPerBlock - 1 && next == pg + 1);
-        if (p.num_pages >= kPagesPerBlock && (run & 0x7fu) == 0x7fu) {
-          const int pg0 = __shfl_sync(0xffffffffu, pg, 0);
+        const bool one = p.num_pages >= kPagesPerBlock && (run & 0x7fu) == 0x7fu;
+        const int boxes = one ? 1 : kPagesPerBlock;
+#pragma unroll 1
+        for (int i = 0; i < boxes; ++i) {
+          const int pgi = __shfl_sync(0xffffffffu, pg, i);
+#pragma unroll
           for (int c = 0; c < L::kChunks; ++c)
-            tma_load_4d_elect(dst + c * L::kChunkBytes, run_map, b, c * 64, g, 0, pg0);
-        } else {
-          for (int i = 0; i < kPagesPerBlock; ++i) {
-            const int pgi = __shfl_sync(0xffffffffu, pg, i);
-            for (int c = 0; c < L::kChunks; ++c)
-              tma_load_4d_elect(dst + c * L::kChunkBytes + i * kPage * 128, page_map, b, c * 64, g,
-                                0, pgi);
-          }
-        }
-      };
-      if (is_k) {  // the unit's Q tile: tokens [tok0, tok0 + 128 / G), heads of KV head g
-        const int e = jbase + k, s = e % L::kKStages;
-        if (e >= L::kKStages && !(ok = wait_bar(sh.k_empty[s], ((e / L::kKStages) - 1) & 1)))
-          break;
-        mbar_arrive_expect_tx_elect(bar(sh.k_full[s]), L::kTileBytes);
-        for (int c = 0; c < L::kChunks; ++c)
-          tma_load_3d_elect(sbase + L::kK + s * L::kTileBytes + c * L::kChunkBytes, &tm_q,
-                            bar(sh.k_full[s]), c * 64, g * G, M.tok0);
-        issued_k = e + 1;
-      }
-      for (int j = 0; j < nb; ++j) {
-        const int jg = jbase + j;
-        const int pid = prefix_pid(blk_lo + j);
-        if (is_k) {
-          const int e = jg + k + 1, s = e % L::kKStages;
-          if (e >= L::kKStages && !(ok = wait_bar(sh.k_empty[s], ((e / L::kKStages) - 1) & 1)))
-            break;
-          load_block(blk_lo + j, pid, sbase + L::kK + s * L::kTileBytes, bar(sh.k_full[s]), &tm_k,
-                     &tm_kc, &tm_k8);
-          issued_k = e + 1;
-        } else {
-          const int s = jg % L::kVStages;
-          if (jg >= L::kVStages &&
-              !(ok = wait_bar(sh.v_empty[s], ((jg / L::kVStages) - 1) & 1)))
-            break;
-          load_block(blk_lo + j, pid, sbase + L::kV + s * L::kTileBytes, bar(sh.v_full[s]), &tm_v,
-                     &tm_vc, &tm_v8);
-          issued_v = jg + 1;
+            tma_load_4d_elect(dst + c * L::kChunkBytes + i * kPage * 128, one ? run_map : page_map,
+                              b, c * 64, g, 0, pgi);
         }
       }
       if (!ok) break;
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(sh.meta_empty[slot]));
-      jbase += nb;
     }
     if (!ok && lane == 0) set_abort(sh, p.err);
     // Do not exit while a copy into this CTA's shared memory is in flight:
     // wait for the most recent phase of every barrier a copy may complete.
-    for (int jg = max(0, issued_k - L::kKStages); jg < issued_k; ++jg)
-      mbar_wait(bar(sh.k_full[jg % L::kKStages]), (jg / L::kKStages) & 1);
-    for (int jg = max(0, issued_v - L::kVStages); jg < issued_v; ++jg)
-      mbar_wait(bar(sh.v_full[jg % L::kVStages]), (jg / L::kVStages) & 1);
+    for (int e = max(0, issued - L::kKStages); e < issued; ++e)
+      mbar_wait(bar(full[e % L::kKStages]), (e / L::kKStages) & 1);
   } else if (warp == 1) {
     // ------------------------------------------------------ MMA issuer --
     // The whole warp runs this loop with warp-uniform values; one elected
@@ -687,12 +666,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         R.blk_lo = M.blk_lo;
         R.nP = M.nP;
         R.valid = r_in < M.nrows;
-        const int token = M.tok0 + r_in / G;
-        const int bl = R.valid ? token / m - M.b_lo : 0;
+        const int rt = p.div_G(r_in), token = M.tok0 + rt;
+        const int bl = R.valid ? p.div_m(token) - M.b_lo : 0;
         R.lim_p = R.valid ? M.fork[bl] : 0;
         R.ps = R.valid ? M.page_start[bl] : 0;
         R.last = R.valid ? M.blen[bl] - m + (token - (M.b_lo + bl) * m) : -1;
-        R.pair = static_cast<size_t>(token) * p.H_q + R.g * G + r_in % G;
+        R.pair = static_cast<size_t>(token) * p.H_q + R.g * G + r_in - rt * G;
       }
       __syncwarp();
       if (R.unit && lane == 0) mbar_arrive(bar(sh.meta_empty[slot]));

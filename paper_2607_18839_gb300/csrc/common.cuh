@@ -34,6 +34,24 @@ struct Plan {
   size_t bytes;      // total workspace bytes
 };
 
+// Division of 0 <= n < 2^31 by a value fixed per call, as a multiplication:
+// with 2^(s-1) < d <= 2^s and mul = ceil(2^(31+s) / d), the error
+// mul * d - 2^(31+s) is below 2^s, so n * mul >> (31 + s) is exact.  (An
+// integer division is some 25 instructions, and code that a CTA runs once is
+// bound by fetching it.)
+struct FastDiv {
+  uint32_t mul, shift;
+  __host__ void set(int d) {
+    uint32_t s = 0;
+    while ((1ll << s) < d) ++s;
+    shift = 31 + s;
+    mul = static_cast<uint32_t>(((1ull << shift) + d - 1) / d);
+  }
+  __host__ __device__ int operator()(int n) const {
+    return static_cast<int>((static_cast<uint64_t>(static_cast<uint32_t>(n)) * mul) >> shift);
+  }
+};
+
 // Kernel parameters of the two attention stages (prefix and suffix).
 struct AttnParams {
   const __nv_bfloat16 *q;
@@ -59,6 +77,8 @@ struct AttnParams {
   int *unit_ctr;        // [2] persistent-kernel unit counter and finished-CTA count, zero between calls
   int n_units;          // work units of the tcgen05 kernel (row tile x KV head x split)
   const int *unit_order;  // the order in which to take them (null: index order)
+  FastDiv div_m, div_G, div_Hkv, div_S;  // by m, G, H_kv and S_p
+  FastDiv div_tile;      // by the tokens of a row tile
   __nv_bfloat16 *out;   // final output, written by the suffix stage
   bool out_align32;     // out is 32-byte aligned (256-bit stores)
   float *lse;           // final lse (may be null)
@@ -111,10 +131,14 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, int sr
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src),
                "r"(src_bytes));
 }
+// 4-byte async global->shared copy.
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
 __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t &r0, uint32_t &r1,

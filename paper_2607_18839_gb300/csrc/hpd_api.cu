@@ -284,6 +284,11 @@ hpd_status hpd_branch_attn_marked(const hpd_branch_attn_args *a, hpd_stream_t st
   p.counters = reinterpret_cast<int *>(ws + pl.off_ctr);
   p.unit_ctr = reinterpret_cast<int *>(ws + pl.off_err + 8);  // header: err word, then counters
   p.n_units = pl.tiles_max * a->H_kv * pl.S_p;
+  p.div_m.set(a->m);
+  p.div_G.set(pl.G);
+  p.div_Hkv.set(a->H_kv);
+  p.div_S.set(pl.S_p);
+  p.div_tile.set(std::max(1, kTcTileRows / pl.G));
   p.unit_order = pl.lpt ? reinterpret_cast<int *>(ws + pl.off_order) : nullptr;
   p.out = static_cast<__nv_bfloat16 *>(a->out);
   p.out_align32 = aligned(a->out, 32);

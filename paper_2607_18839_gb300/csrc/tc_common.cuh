@@ -50,49 +50,43 @@ __device__ __forceinline__ float softmax_half_tmem(uint32_t s_addr, int h, int l
   float mx = NEG_INF;
   // A positive scale keeps the order of the scores, so the maximum can be
   // taken over the raw scores and an invisible score can simply become -inf
-  // in place (its exponential is then 0): one select per score instead of a
-  // visibility test in both loops below.
+  // in place (its exponential is then 0): one select per score and no
+  // visibility test in the two loops below.  Another scale is applied to the
+  // scores first.
   const bool raw = sl2 > 0.f;
+  const float mul = raw ? sl2 : 1.f;
   if (!all_empty) {
     tmem_ld32(s_addr + h * kH, v);
     tmem_ld32(s_addr + h * kH + 32, v + 32);
     tmem_ld_wait();
+    if (!raw) {
+#pragma unroll
+      for (int c = 0; c < kH; ++c) v[c] = __float_as_uint(__uint_as_float(v[c]) * sl2);
+    }
+    if (!all_full) {
+      // bit c of vis: column c of this half is visible
+      auto below = [](int n) -> uint64_t {
+        return n <= 0 ? 0ull : n >= 64 ? ~0ull : (1ull << n) - 1ull;
+      };
+      const uint64_t vis = below(hi) & ~below(lo);
+      const uint32_t vis0 = static_cast<uint32_t>(vis), vis1 = static_cast<uint32_t>(vis >> 32);
+#pragma unroll
+      for (int c = 0; c < 32; ++c) {
+        v[c] = (vis0 & (1u << c)) ? v[c] : 0xff800000u;
+        v[c + 32] = (vis1 & (1u << c)) ? v[c + 32] : 0xff800000u;
+      }
+    }
     float mx8[8];
 #pragma unroll
     for (int a = 0; a < 8; ++a) mx8[a] = NEG_INF;
-    if (raw) {
-      if (!all_full) {
-        // bit c of vis: column c of this half is visible
-        auto below = [](int n) -> uint64_t {
-          return n <= 0 ? 0ull : n >= 64 ? ~0ull : (1ull << n) - 1ull;
-        };
-        const uint64_t vis = below(hi) & ~below(lo);
-        const uint32_t vis0 = static_cast<uint32_t>(vis), vis1 = static_cast<uint32_t>(vis >> 32);
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
-          v[c] = (vis0 & (1u << c)) ? v[c] : 0xff800000u;
-          v[c + 32] = (vis1 & (1u << c)) ? v[c + 32] : 0xff800000u;
-        }
-      }
+    for (int c = 0; c < kH; c += 16)
 #pragma unroll
-      for (int c = 0; c < kH; c += 16)
-#pragma unroll
-        for (int a = 0; a < 8; ++a)
-          mx8[a] = fmax3(mx8[a], __uint_as_float(v[c + 2 * a]), __uint_as_float(v[c + 2 * a + 1]));
-    } else {
-#pragma unroll
-      for (int c = 0; c < kH; c += 16)
-#pragma unroll
-        for (int a = 0; a < 8; ++a) {
-          const int c0 = c + 2 * a;
-          const float x0 = c0 >= lo && c0 < hi ? __uint_as_float(v[c0]) * sl2 : NEG_INF;
-          const float x1 = c0 + 1 >= lo && c0 + 1 < hi ? __uint_as_float(v[c0 + 1]) * sl2 : NEG_INF;
-          mx8[a] = fmax3(mx8[a], x0, x1);
-        }
-    }
+      for (int a = 0; a < 8; ++a)
+        mx8[a] = fmax3(mx8[a], __uint_as_float(v[c + 2 * a]), __uint_as_float(v[c + 2 * a + 1]));
     mx = fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]),
-               fmaxf(mx8[6], mx8[7]));
-    if (raw) mx *= sl2;
+               fmaxf(mx8[6], mx8[7])) *
+         mul;
   }
   mx = xchg(mx);
   const float m_new = mx > m_run + kRescaleLog2 ? mx : m_run;
@@ -106,40 +100,22 @@ __device__ __forceinline__ float softmax_half_tmem(uint32_t s_addr, int h, int l
     tmem_st16(s_addr + h * 32, pk);
     tmem_st16(s_addr + h * 32 + 16, pk);
   } else {
-    const float2 sl2x2 = make_float2(sl2, sl2), nbase2 = make_float2(-base, -base);
+    const float2 mul2 = make_float2(mul, mul), nbase2 = make_float2(-base, -base);
     float2 sum4[4];
 #pragma unroll
     for (int a = 0; a < 4; ++a) sum4[a] = make_float2(0.f, 0.f);
-    if (all_full || raw) {
 #pragma unroll
-      for (int ch = 0; ch < 2; ++ch) {
+    for (int ch = 0; ch < 2; ++ch) {
 #pragma unroll
-        for (int c = 0; c < 32; c += 2) {
-          const int col = ch * 32 + c;
-          const float2 x = make_float2(__uint_as_float(v[col]), __uint_as_float(v[col + 1]));
-          const float2 arg = __ffma2_rn(x, sl2x2, nbase2);
-          const float2 e = make_float2(fast_exp2(arg.x), fast_exp2(arg.y));
-          sum4[(c >> 1) & 3] = __fadd2_rn(sum4[(c >> 1) & 3], e);
-          pk[c / 2] = pack_bf16x2(e.x, e.y);
-        }
-        tmem_st16(s_addr + h * 32 + ch * 16, pk);
+      for (int c = 0; c < 32; c += 2) {
+        const int col = ch * 32 + c;
+        const float2 x = make_float2(__uint_as_float(v[col]), __uint_as_float(v[col + 1]));
+        const float2 arg = __ffma2_rn(x, mul2, nbase2);
+        const float2 e = make_float2(fast_exp2(arg.x), fast_exp2(arg.y));
+        sum4[(c >> 1) & 3] = __fadd2_rn(sum4[(c >> 1) & 3], e);
+        pk[c / 2] = pack_bf16x2(e.x, e.y);
       }
-    } else {
-#pragma unroll
-      for (int ch = 0; ch < 2; ++ch) {
-#pragma unroll
-        for (int c = 0; c < 32; c += 2) {
-          const int col = ch * 32 + c;
-          const float2 x = make_float2(__uint_as_float(v[col]), __uint_as_float(v[col + 1]));
-          const float2 arg = __ffma2_rn(x, sl2x2, nbase2);
-          float2 e;
-          e.x = col >= lo && col < hi ? fast_exp2(arg.x) : 0.f;
-          e.y = col + 1 >= lo && col + 1 < hi ? fast_exp2(arg.y) : 0.f;
-          sum4[(c >> 1) & 3] = __fadd2_rn(sum4[(c >> 1) & 3], e);
-          pk[c / 2] = pack_bf16x2(e.x, e.y);
-        }
-        tmem_st16(s_addr + h * 32 + ch * 16, pk);
-      }
+      tmem_st16(s_addr + h * 32 + ch * 16, pk);
     }
     const float2 s01 = __fadd2_rn(sum4[0], sum4[1]), s23 = __fadd2_rn(sum4[2], sum4[3]);
     const float2 s03 = __fadd2_rn(s01, s23);

@@ -421,3 +421,17 @@ def test_accept_misaligned_rows(hpd):
     tok, acc = run_accept(hpd, logits, np.zeros((9, 7), np.int32))
     np.testing.assert_array_equal(tok, ref_tok)
     np.testing.assert_array_equal(acc, ref_acc)
+
+
+@pytest.mark.parametrize("scale", [-0.2, 1e-3])
+def test_parity_scale_that_reverses_or_flattens_the_scores(hpd, scale):
+    # a scale that is not positive takes the scores' own path through the
+    # softmax (they are scaled before the masks and the maximum): partly
+    # visible prefix and suffix blocks, full ones, rows without private keys;
+    # same bounds as every parity case (the scores stay below 64 in size)
+    inp = W.build_inputs([300, 130], [3, 2], [0, 5, 40, 130, 17], 3, 16, 2, 128, seed=51,
+                         branch_prefix_len=[300, 129, 7, 130, 128], scale=scale)
+    ref_out, ref_lse = oracle.branch_attn(inp)
+    out, lse, err = run_gpu(hpd, inp)
+    assert err == 0
+    compare(inp, out, lse, ref_out, ref_lse)
