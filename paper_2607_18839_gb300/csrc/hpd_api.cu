@@ -52,6 +52,29 @@ hpd_status check_scalars(const hpd_branch_attn_args *a) {
   return HPD_OK;
 }
 
+// Head ratios G that do not divide 128 run on the tcgen05 kernel too (row
+// tiles of 128 / G whole tokens), except where the warp-MMA stages measured
+// faster: a packed suffix block serves the m G rows of a branch only, so
+// where private keys dominate the masked rows cost more than the tensor cores
+// gain.  The rule compares a tile's suffix blocks (at the page table's width)
+// with its prefix blocks.  us per call, warp MMA / tcgen05, branches x prefix
+// / private tokens up to:
+//   m G = 3   64 x 1,024 / 1,024  45 / 108;  16 x 1,024 / 64     24.6 / 16.4
+//   m G = 7   64 x 1,024 / 1,024  52 / 58
+//   m G = 10  16 x 2,000 / 100    33 / 20
+//   m G = 12  256 x 1,024 / 1,024  102 / 68;  64 x 64 / 1,024    40 / 58
+//   m G = 14  32 x 100 / 2,048    52 / 66;  256 x 1,024 / 512    119 / 63
+// A call of up to 32 stacked rows keeps the launch plan it reports.
+constexpr int kMmaMaxRows = 32;
+bool tc_ragged(const hpd_branch_attn_args *a, int G, int maxP) {
+  const int rows = a->m * G;
+  if (static_cast<long long>(a->B) * rows <= kMmaMaxRows) return false;
+  const int tile_branches = std::min(a->B, ceil_div(kTcTileRows, rows));
+  const long long suffix =
+      ceil_div(static_cast<long long>(tile_branches) * a->max_pages_per_branch, 8);
+  return suffix <= (rows >= 12 ? 16ll : 1ll) * ceil_div(maxP, 128);
+}
+
 hpd::Plan make_plan(const hpd_branch_attn_args *a) {
   hpd::Plan pl{};
   pl.G = a->H_q / a->H_kv;
@@ -60,11 +83,12 @@ hpd::Plan make_plan(const hpd_branch_attn_args *a) {
                                    : a->prefix_tokens;
   if (a->prefix_page_table)
     maxP = static_cast<int>(std::min<long long>(maxP, 16LL * a->max_prefix_pages));
-  pl.use_tc = (a->D == 64 || a->D == 128) && (kTcTileRows % pl.G == 0);
+  const bool divides = kTcTileRows % pl.G == 0;
+  const int tile_tokens = kTcTileRows / pl.G;  // rows past tile_tokens * G stay unused
+  pl.use_tc = divides || tc_ragged(a, pl.G, maxP);
   if (pl.use_tc) {
     // tcgen05 kernel: units of 128 stacked rows (128 / G tokens) of one
     // page and KV head, one CTA per SM taking units in turn.
-    const int tile_tokens = kTcTileRows / pl.G;
     const int tiles = ceil_div(static_cast<long long>(a->B) * a->m, tile_tokens);
     pl.tiles_max = tiles + a->n_docs;
     // Key splits: minimise the estimated time of the step, i.e. waves of
@@ -102,30 +126,44 @@ hpd::Plan make_plan(const hpd_branch_attn_args *a) {
                           block_us / kPlanSms;
     pl.lpt = ctas * best >= kLptWaves * kPlanSms && est_us >= kLptMinUs &&
              hpd::unit_order_smem_bytes(a->n_docs, a->B, pl.tiles_max) <= kOrderSmemMax;
-  } else {
+  }
+  int mma_splits = 1;
+  if (!divides) {
     const long long stacked = static_cast<long long>(a->B) * a->m * pl.G;
     const int tiles = ceil_div(stacked, kPrefixTileRows);
-    pl.tiles_max = tiles + a->n_docs;
     const long long tiles_est = static_cast<long long>(std::max(tiles, 1)) * a->H_kv;
     int sp = ceil_div(kTargetCtas, tiles_est);
     sp = std::min(sp, std::max(1, ceil_div(maxP, 256)));
-    pl.S_p = std::max(1, std::min(sp, kMaxPrefixSplits));
+    mma_splits = std::max(1, std::min(sp, kMaxPrefixSplits));
+    if (!pl.use_tc) {
+      pl.tiles_max = tiles + a->n_docs;
+      pl.S_p = mma_splits;
+    }
   }
   const int maxL = a->max_pages_per_branch * hpd::kPage;
   pl.S_s = std::max(1, std::min(ceil_div(maxL, kSuffixSplitKeys), kMaxSuffixSplits));
   const int rows_s = a->m * pl.G;
   pl.wr_s = rows_s <= 16 ? 1 : (rows_s <= 32 ? 2 : 4);
   pl.rt_s = ceil_div(rows_s, 16 * pl.wr_s);
-  const size_t S = static_cast<size_t>(pl.S_p + pl.S_s);
+  // With a head ratio that does not divide 128 the workspace is sized for the
+  // warp-MMA stages whichever path runs (its size is part of the interface: a
+  // caller's buffer, the limit of the built-in array).  Their partials, at
+  // least two, hold the tcgen05 kernel's splits or, unsplit, its unit order.
+  const size_t S = static_cast<size_t>((divides ? pl.S_p : mma_splits) + pl.S_s);
+  if (!divides && pl.use_tc) pl.S_p = std::min(pl.S_p, static_cast<int>(S));
   const size_t pairs = static_cast<size_t>(pl.rows_total) * a->H_q;
   pl.off_err = 0;
   pl.off_ctr = kAlign;
   pl.off_opart = align_up(pl.off_ctr + static_cast<size_t>(a->B) * a->H_kv * pl.rt_s * sizeof(int));
   pl.off_lpart = align_up(pl.off_opart + S * pairs * a->D * sizeof(float));
   pl.off_order = align_up(pl.off_lpart + S * pairs * sizeof(float));
-  const size_t n_units =
-      pl.use_tc ? static_cast<size_t>(std::max(pl.tiles_max, 0)) * a->H_kv * pl.S_p : 0;
-  pl.bytes = align_up(pl.off_order + n_units * sizeof(int));
+  const size_t order_bytes =
+      pl.use_tc ? static_cast<size_t>(std::max(pl.tiles_max, 0)) * a->H_kv * pl.S_p * sizeof(int) : 0;
+  pl.bytes = align_up(pl.off_order + (divides ? order_bytes : 0));
+  if (!divides) {
+    pl.off_order = pl.off_opart;
+    pl.lpt = pl.lpt && pl.S_p == 1 && pl.off_order + order_bytes <= pl.bytes;
+  }
   return pl;
 }
 
@@ -288,7 +326,7 @@ hpd_status hpd_branch_attn_marked(const hpd_branch_attn_args *a, hpd_stream_t st
   p.div_G.set(pl.G);
   p.div_Hkv.set(a->H_kv);
   p.div_S.set(pl.S_p);
-  p.div_tile.set(std::max(1, kTcTileRows / pl.G));
+  p.div_tile.set(kTcTileRows / pl.G);
   p.unit_order = pl.lpt ? reinterpret_cast<int *>(ws + pl.off_order) : nullptr;
   p.out = static_cast<__nv_bfloat16 *>(a->out);
   p.out_align32 = aligned(a->out, 32);

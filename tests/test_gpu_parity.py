@@ -435,3 +435,22 @@ def test_parity_scale_that_reverses_or_flattens_the_scores(hpd, scale):
     out, lse, err = run_gpu(hpd, inp)
     assert err == 0
     compare(inp, out, lse, ref_out, ref_lse)
+
+
+@pytest.mark.parametrize("hq,hkv,m,D", [(6, 2, 4, 128), (10, 2, 5, 64), (28, 4, 2, 128), (15, 1, 1, 64),
+                                        (44, 4, 16, 128)])
+def test_ratio_that_does_not_divide_the_tile(hpd, hq, hkv, m, D):
+    # row tiles of 128 / G whole tokens (126, 125, 126, 120 and 121 rows): the
+    # unused rows, tiles that end inside a branch, a page whose last tile has
+    # one token, several pages, fork lengths; same bounds as every parity case
+    tt = 128 // (hq // hkv)
+    n = max(2, -(-(tt + 1) // m))  # branches of the first page: just over one tile
+    inp = W.build_inputs([1500, 700], [n, 3], [(7 * b) % 90 for b in range(n + 3)], m, hq, hkv, D,
+                         seed=52, branch_prefix_len=[1500 - 3 * b for b in range(n)] + [700, 0, 699])
+    op = hpd.BranchAttn(hpd.DeviceInputs.from_host(inp))
+    assert hpd.hpd_branch_attn_kernel_name(op.args, 0) == "branch_attn_tc"
+    ref_out, ref_lse = oracle.branch_attn(inp)
+    for paged in (False, True):
+        out, lse, err = run_gpu(hpd, W.page_the_prefix(inp, seed=95) if paged else inp)
+        assert err == 0
+        compare(inp, out, lse, ref_out, ref_lse)
