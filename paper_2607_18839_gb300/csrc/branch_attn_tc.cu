@@ -50,10 +50,13 @@
 //               128 key columns and half of O's columns; thread t of warp w
 //               owns TMEM lane 32*(w%4)+t, i.e. one query row.  The two
 //               halves of a row exchange their partial max through shared
-//               memory.  O is rescaled in TMEM only when a row's running
-//               max grows by more than 2^8; the stale max stays exact after
-//               the final normalisation.  At a unit change they only read
-//               the next unit's metadata before the epilogue.
+//               memory only in the first block that some row of the warp
+//               sees keys of: that maximum is the row's base, and later
+//               blocks take their exponentials against it without waiting
+//               for anything.  Should a score exceed its base by more than
+//               2^64, the unit runs once more with running maxima in every
+//               block (O then rescaled in TMEM when one grows by more than
+//               2^8), and so do the CTA's later units.
 // One split: the unit writes the final bf16 output and lse.  Several splits:
 // it writes its normalised fp32 partial and lse for merge.cu.
 // Code size: every CTA fetches the kernel's instructions anew, at some 150
@@ -106,6 +109,7 @@ struct UnitMeta {
   int n_blocks;  // blocks of the split (> 0)
   int doc;       // page (document) of the tile
   int pp_last;   // paged prefix: last prefix page any row of the tile sees
+  int exact;     // every block's base is the running maximum
   int page_start[kMaxUnitBranches + 1];  // packed page offset of each branch
   int blen[kMaxUnitBranches];            // private length L_b (clamped)
   int fork[kMaxUnitBranches];            // prefix keys visible to the branch
@@ -147,6 +151,12 @@ struct __align__(8) TcShared {
   float xmax[2][2][kRows];  // [half][block parity][row]
   float xsum[2][kRows];     // [half][row]
   int xseq[2][2][4];        // [max | sum][half][quadrant]
+  // units (by number in this CTA, modulo 32) whose scores left the window of
+  // their base and that run once more, with running maxima
+  unsigned redo;
+  int exact;         // set with the first of them: later units run so at once
+  int units_done;    // softmax warps that finished a unit's epilogue
+  int unit_id[32];   // the last units issued
 };
 
 __device__ __forceinline__ void set_abort(TcShared &sh, uint32_t *err) {
@@ -186,6 +196,16 @@ __device__ __forceinline__ bool await_seq(const int *flag, int seq, const TcShar
   return load_seq(flag) >= seq || await_seq_slow(flag, seq, &sh.abort);
 }
 
+// Wait (bounded, mostly asleep) until `n` epilogues of softmax warps are done.
+__device__ __noinline__ bool await_units(int n, const TcShared &sh) {
+  const uint64_t t0 = globaltimer();
+  while (load_seq(&sh.units_done) < n) {
+    if (aborted(sh) || globaltimer() - t0 > kWaitLimitNs) return false;
+    __nanosleep(100);
+  }
+  return true;
+}
+
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
     branch_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k,
@@ -214,6 +234,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   // ------------------------------------------------------ once per CTA --
   if (tid == 0) {
     sh.abort = 0;
+    sh.redo = 0u;
+    sh.exact = 0;
+    sh.units_done = 0;
     for (int s = 0; s < kMaxRing; ++s) {
       mbar_init(bar(sh.k_full[s]), 1);
       mbar_init(bar(sh.v_full[s]), 1);
@@ -248,6 +271,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ------------------------------------------------------- scheduler --
     // Fills slot k & 1 with the k-th unit of this CTA that has keys; units
     // without any get their output written here and are skipped.
+    unsigned redo = 0;  // units to run once more
+    auto take_redo = [&] {
+      unsigned r = 0;
+      if (lane == 0) r = atomicExch(&sh.redo, 0u);
+      return __shfl_sync(0xffffffffu, r, 0);
+    };
     for (int k = 0;; ++k) {
       const int slot = k & 1;
       if (k >= 2 && !wait_bar(sh.meta_empty[slot], ((k >> 1) - 1) & 1)) {
@@ -258,10 +287,25 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool have = false;
       for (;;) {
         int u = 0;
-        if (lane == 0) u = atomicAdd(p.unit_ctr, 1);
-        u = __shfl_sync(0xffffffffu, u, 0);
-        if (u >= p.n_units || aborted(sh)) break;
-        if (p.unit_order) u = p.unit_order[u];  // longest units first
+        if (!redo && *static_cast<volatile unsigned *>(&sh.redo)) redo = take_redo();
+        const bool again = redo != 0;
+        if (again) {
+          u = sh.unit_id[__ffs(redo) - 1];
+          redo &= redo - 1;
+        } else {
+          if (lane == 0) u = atomicAdd(p.unit_ctr, 1);
+          u = __shfl_sync(0xffffffffu, u, 0);
+          if (aborted(sh)) break;
+          if (u >= p.n_units) {
+            // none left, once the units still running need no second pass
+            if (!__all_sync(0xffffffffu, await_units(kSoftmaxWarps * k, sh))) break;
+            redo = take_redo();
+            if (!redo) break;
+            continue;
+          }
+          if (p.unit_order) u = p.unit_order[u];  // longest units first
+        }
+        const int u_id = u;
         const int us = p.div_S(u), split = u - us * p.S_p;
         const int tile = p.div_Hkv(us), g = us - tile * p.H_kv;
         // the page owning the tile: page d has ceil(#branches(d) * m / TT) tiles
@@ -401,6 +445,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           M.pp_last = max(kmax - 1, 0) / kPage;
           M.blk_lo = blk_lo;
           M.n_blocks = blk_hi - blk_lo;
+          M.exact = again || *static_cast<volatile int *>(&sh.exact);
+          sh.unit_id[k & 31] = u_id;
         }
         have = true;
         break;
@@ -552,7 +598,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (issuer) {
 #pragma unroll
         for (int kk = 0; kk < kBlk / 16; ++kk)
-          mma_ts_one(tmem + L::kColO, tmem + pcol + kk * 8, vd + ((kk * 16 * 128) >> 4), idesc_pv,
+          mma_ts_one(tmem + L::kColO, tmem + pcol + kk * 8 + (kk >= 4 ? 32 : 0), vd + ((kk * 16 * 128) >> 4), idesc_pv,
                      (!first || kk > 0) ? 1u : 0u);
       }
       __syncwarp();
@@ -598,6 +644,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool ok = true, k_ready = false;
     for (int k = 0; ok; ++k) {
       const int slot = k & 1;
+      // no next unit yet: the scheduler may be waiting for this one's end
+      if (has_pend && !__all_sync(0xffffffffu, mbar_test_wait(bar(sh.meta_full[slot]), (k >> 1) & 1))) {
+        if (!(ok = do_pv(pend, -1, k_ready))) break;
+        has_pend = false;
+      }
       if (!(ok = wait(sh.meta_full[slot], (k >> 1) & 1))) break;
       const bool valid = meta[slot].valid != 0;
       const int nb = meta[slot].n_blocks;
@@ -647,7 +698,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // j <= last, which start at packed page ps).
     struct Row {
       bool unit;  // false: no unit left
-      bool valid;
+      bool valid, exact;
       int g, split, nb, blk_lo, nP, lim_p, ps, last;
       size_t pair;
     };
@@ -666,6 +717,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         R.blk_lo = M.blk_lo;
         R.nP = M.nP;
         R.valid = r_in < M.nrows;
+        R.exact = M.exact != 0;
         const int rt = p.div_G(r_in), token = M.tok0 + rt;
         const int bl = R.valid ? p.div_m(token) - M.b_lo : 0;
         R.lim_p = R.valid ? M.fork[bl] : 0;
@@ -679,16 +731,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
     const uint32_t o_col = L::kColO + h * (D / 2);
     int jbase = 0;
-    Row cur{}, nxt{};
-    bool ok = begin_unit(0, cur);
-    for (int k = 0; ok && cur.unit; ++k) {
+    Row cur{};
+    bool ok = true;
+    for (int k = 0; ok; ++k) {
+      if (!(ok = begin_unit(k, cur)) || !cur.unit) break;
       float m_run = NEG_INF, l_half = 0.f;
+      bool inside = true;  // the scores stay in the window of their base
       for (int j = 0; j < cur.nb; ++j) {
         const int jg = jbase + j;
         const int si = jg & 1;
-        // warp-uniform outcome: the tcgen05.ld / st below are warp-collective
-        if (!(ok = wait_bar(sh.s_full[si], (jg >> 1) & 1))) break;
-        tc_fence_after();
         const int jb = cur.blk_lo + j;
         int lo, hi;
         if (jb < cur.nP) {
@@ -699,26 +750,38 @@ __global__ void __launch_bounds__(kThreads, 1)
           lo = max(0, off);
           hi = min(kBlk, off + cur.last + 1);
         }
-        const int par = jg & 1;
-        bool xok = true;
-        auto xchg = [&](float mx) {
-          sh.xmax[h][par][r_in] = mx;
-          tc_fence_before();
-          publish_seq(&sh.xseq[0][h][quad], jg + 1);
-          xok = await_seq(&sh.xseq[0][h ^ 1][quad], jg + 1, sh);
-          tc_fence_after();
-          return fmaxf(mx, sh.xmax[h ^ 1][par][r_in]);
-        };
-        const float alpha =
-            tc::softmax_half_tmem(t_lane + L::col_s(si), h, lo, hi, sl2, m_run, l_half, xchg);
-        if (!(ok = __all_sync(0xffffffffu, xok))) break;
+        // A row's base is the maximum of the first block it sees keys of;
+        // both halves come to the same answer here, and take that block's
+        // maximum together.  (exact: every block's.)
+        const bool find_max =
+            cur.exact || __any_sync(0xffffffffu, m_run == NEG_INF && min(hi, kBlk) > lo);
+        // warp-uniform outcome: the tcgen05.ld / st below are warp-collective
+        if (!(ok = wait_bar(sh.s_full[si], (jg >> 1) & 1))) break;
+        tc_fence_after();
+        const uint32_t s_addr = t_lane + L::col_s(si) + h * 64;
+        bool rescale = false;
+        float alpha = 1.f;
+        if (!find_max) {
+          inside &= tc::softmax_half_based(s_addr, lo - h * 64, hi - h * 64, sl2, m_run, l_half);
+        } else {
+          const int par = jg & 1;
+          bool xok = true;
+          auto xchg = [&](float mx) {
+            sh.xmax[h][par][r_in] = mx;
+            publish_seq(&sh.xseq[0][h][quad], jg + 1);
+            xok = await_seq(&sh.xseq[0][h ^ 1][quad], jg + 1, sh);
+            return fmaxf(mx, sh.xmax[h ^ 1][par][r_in]);
+          };
+          alpha = tc::softmax_half_max(s_addr, lo - h * 64, hi - h * 64, sl2, m_run, l_half, xchg);
+          if (!(ok = __all_sync(0xffffffffu, xok))) break;
+          rescale = __any_sync(0xffffffffu, j > 0 && alpha != 1.f);
+        }
         // Before O may be rescaled, the P V MMA of block jg-1 must have
         // landed: a warp that rescales waits for it.  Warps skip the wait
         // when they do not rescale, yet the parity test stays exact: Q K^T
         // (jg) was issued after P V (jg-2), so the S commit awaited above
         // implies P V (jg-2) has completed, and P V (jg) needs this block's
         // P; the barrier is in one of two consecutive phases.
-        const bool rescale = __any_sync(0xffffffffu, j > 0 && alpha != 1.f);
         if (rescale) {
           if (!(ok = wait_bar(sh.pv_done, (jg - 1) & 1))) break;
           tc_fence_after();
@@ -738,9 +801,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) mbar_arrive(bar(sh.p_full[si]));
       }
       if (!ok) break;
-      // the next unit's Q goes to TMEM before this unit's epilogue, so that
-      // its first Q K^T MMAs run meanwhile
-      if (!(ok = begin_unit(k + 1, nxt))) break;
+      if (__any_sync(0xffffffffu, !inside && cur.valid)) {
+        if (lane == 0) {
+          atomicOr(&sh.redo, 1u << (k & 31));
+          atomicExch(&sh.exact, 1);
+        }
+      }
       // ---------------------------------------------------- epilogue --
       // row sum over both halves
       sh.xsum[h][r_in] = l_half;
@@ -793,9 +859,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       // O may be overwritten by the next unit once every warp has read it
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar(sh.o_empty));
+      if (lane == 0) {
+        mbar_arrive(bar(sh.o_empty));
+        __threadfence_block();
+        atomicAdd(&sh.units_done, 1);
+      }
       jbase += cur.nb;
-      cur = nxt;
     }
     if (!ok && lane == 0) set_abort(sh, p.err);
   }

@@ -23,107 +23,135 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
 constexpr int kRows = 128;  // stacked query rows of one tile (MMA M)
 constexpr int kBlk = 128;   // keys per block (MMA N of S = Q K^T)
 constexpr float kRescaleLog2 = 8.0f;  // tolerate a stale row max up to 2^8
+constexpr float kWindowLog2 = 64.0f;  // scores this far above a fixed base stay far from overflow
 
-// Half of one 128-key block of a row's online softmax: this thread owns the
-// 64 columns [64 h, 64 h + 64) of its row; the thread of the other half (the
-// same TMEM lane, another warpgroup) owns the rest.  s_addr is this thread's
-// lane at the block's first column; lo / hi bound the row's visible columns
-// in block coordinates.  xchg(max of my visible scaled scores) returns the
-// row max over both halves; it must synchronise the two halves, which also
-// orders every P store of either half after both have read their scores
-// (P half h lands in packed columns [32 h, 32 h + 32), over scores of half 0).
-// Both halves apply the same running max, so O's two column halves and the
-// two partial sums l_half stay consistent.  Returns the rescale factor of O.
-// Warp-collective (tcgen05.ld / st).
+// A key the row does not see gets the score -inf: 32 columns, visible from
+// lo to hi; scale: multiply by mul first.
+__device__ __forceinline__ void mask32(uint32_t *v, int lo, int hi, bool scale, float mul) {
+  auto below = [](int n) -> uint32_t { return n <= 0 ? 0u : n >= 32 ? ~0u : (1u << n) - 1u; };
+  const uint32_t vis = below(hi) & ~below(lo);
+  if (scale) {
+#pragma unroll
+    for (int c = 0; c < 32; ++c) v[c] = __float_as_uint(__uint_as_float(v[c]) * mul);
+  }
+#pragma unroll
+  for (int c = 0; c < 32; ++c) v[c] = (vis & (1u << c)) ? v[c] : 0xff800000u;
+}
+
+// exp2(mul * v - base) of 32 scores as bf16 pairs in TMEM columns [dst, dst +
+// 16); adds to the sums.  With MAX, the maxima of the scores are taken in the
+// same loop (another pipe than the exponentials').
+template <bool MAX>
+__device__ __forceinline__ void exp32(uint32_t dst, const uint32_t *v, float mul, float base,
+                                      float2 *sum4, float *mx4) {
+  const float2 mul2 = make_float2(mul, mul), nbase2 = make_float2(-base, -base);
+  uint32_t pk[16];
+#pragma unroll
+  for (int c = 0; c < 32; c += 2) {
+    const float2 x = make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1]));
+    const float2 arg = __ffma2_rn(x, mul2, nbase2);
+    const float2 e = make_float2(fast_exp2(arg.x), fast_exp2(arg.y));
+    sum4[(c >> 1) & 3] = __fadd2_rn(sum4[(c >> 1) & 3], e);
+    pk[c / 2] = pack_bf16x2(e.x, e.y);
+    if constexpr (MAX) mx4[(c >> 1) & 3] = fmax3(mx4[(c >> 1) & 3], x.x, x.y);
+  }
+  sm100::tmem_st16(dst, pk);
+}
+__device__ __forceinline__ float sum_of(const float2 *sum4) {
+  const float2 s01 = __fadd2_rn(sum4[0], sum4[1]), s23 = __fadd2_rn(sum4[2], sum4[3]);
+  const float2 s03 = __fadd2_rn(s01, s23);
+  return s03.x + s03.y;
+}
+
+// One 128-key block of a row's online softmax is the work of two threads: the
+// one of half h owns the 64 columns [64 h, 64 h + 64) of its row.  s_addr is
+// this thread's lane at the half's first column, where P (bf16 pairs, 32
+// columns) replaces the scores; lo / hi bound the row's visible columns in
+// half-block coordinates.  Both threads use the same base, so that O's two
+// column halves and the two partial sums l_half stay consistent.
+// A positive scale keeps the order of the scores, so the maximum is taken
+// over the raw scores and an invisible one simply becomes -inf in place (its
+// exponential is then 0); another scale is applied to the scores first.
+//
+// softmax_half_max: the base is the running maximum, which xchg(max of my
+// visible scaled scores) takes over both halves (and synchronises them).
+// Returns the rescale factor of O.  Warp-collective (tcgen05.ld / st).
 template <class Xchg>
-__device__ __forceinline__ float softmax_half_tmem(uint32_t s_addr, int h, int lo, int hi,
-                                                   float sl2, float &m_run, float &l_half,
-                                                   Xchg xchg) {
+__device__ __forceinline__ float softmax_half_max(uint32_t s_addr, int lo, int hi, float sl2,
+                                                  float &m_run, float &l_half, Xchg xchg) {
   using namespace sm100;
   const float NEG_INF = -__int_as_float(0x7f800000);
-  constexpr int kH = kBlk / 2;
-  lo = max(lo - h * kH, 0);
-  hi = min(hi - h * kH, kH);
-  const bool all_empty = __all_sync(0xffffffffu, hi <= lo);
-  const bool all_full = __all_sync(0xffffffffu, lo == 0 && hi == kH);
-  uint32_t v[kH];
-  float mx = NEG_INF;
-  // A positive scale keeps the order of the scores, so the maximum can be
-  // taken over the raw scores and an invisible score can simply become -inf
-  // in place (its exponential is then 0): one select per score and no
-  // visibility test in the two loops below.  Another scale is applied to the
-  // scores first.
   const bool raw = sl2 > 0.f;
   const float mul = raw ? sl2 : 1.f;
-  if (!all_empty) {
-    tmem_ld32(s_addr + h * kH, v);
-    tmem_ld32(s_addr + h * kH + 32, v + 32);
-    tmem_ld_wait();
-    if (!raw) {
+  uint32_t v[64];
+  float mx8[8];
 #pragma unroll
-      for (int c = 0; c < kH; ++c) v[c] = __float_as_uint(__uint_as_float(v[c]) * sl2);
-    }
-    if (!all_full) {
-      // bit c of vis: column c of this half is visible
-      auto below = [](int n) -> uint64_t {
-        return n <= 0 ? 0ull : n >= 64 ? ~0ull : (1ull << n) - 1ull;
-      };
-      const uint64_t vis = below(hi) & ~below(lo);
-      const uint32_t vis0 = static_cast<uint32_t>(vis), vis1 = static_cast<uint32_t>(vis >> 32);
+  for (int a = 0; a < 8; ++a) mx8[a] = NEG_INF;
+  tmem_ld32(s_addr, v);
+  tmem_ld32(s_addr + 32, v + 32);
+  tmem_ld_wait32(v);
+  tmem_ld_wait32(v + 32);
+  mask32(v, lo, hi, !raw, sl2);
+  mask32(v + 32, lo - 32, hi - 32, !raw, sl2);
 #pragma unroll
-      for (int c = 0; c < 32; ++c) {
-        v[c] = (vis0 & (1u << c)) ? v[c] : 0xff800000u;
-        v[c + 32] = (vis1 & (1u << c)) ? v[c + 32] : 0xff800000u;
-      }
-    }
-    float mx8[8];
+  for (int c = 0; c < 64; c += 16)
 #pragma unroll
-    for (int a = 0; a < 8; ++a) mx8[a] = NEG_INF;
-#pragma unroll
-    for (int c = 0; c < kH; c += 16)
-#pragma unroll
-      for (int a = 0; a < 8; ++a)
-        mx8[a] = fmax3(mx8[a], __uint_as_float(v[c + 2 * a]), __uint_as_float(v[c + 2 * a + 1]));
-    mx = fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]),
-               fmaxf(mx8[6], mx8[7])) *
-         mul;
-  }
-  mx = xchg(mx);
+    for (int a = 0; a < 8; ++a)
+      mx8[a] = fmax3(mx8[a], __uint_as_float(v[c + 2 * a]), __uint_as_float(v[c + 2 * a + 1]));
+  const float mx = xchg(fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]),
+                              fmaxf(mx8[6], mx8[7])) *
+                        mul);
   const float m_new = mx > m_run + kRescaleLog2 ? mx : m_run;
   const float base = m_new == NEG_INF ? 0.f : m_new;
   const float alpha = m_new == m_run ? 1.f : fast_exp2(m_run - base);
-  float sum = 0.f;
-  uint32_t pk[16];
-  if (all_empty) {
+  float2 sum4[4];
 #pragma unroll
-    for (int c = 0; c < 16; ++c) pk[c] = 0u;
-    tmem_st16(s_addr + h * 32, pk);
-    tmem_st16(s_addr + h * 32 + 16, pk);
-  } else {
-    const float2 mul2 = make_float2(mul, mul), nbase2 = make_float2(-base, -base);
-    float2 sum4[4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) sum4[a] = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int ch = 0; ch < 2; ++ch) {
-#pragma unroll
-      for (int c = 0; c < 32; c += 2) {
-        const int col = ch * 32 + c;
-        const float2 x = make_float2(__uint_as_float(v[col]), __uint_as_float(v[col + 1]));
-        const float2 arg = __ffma2_rn(x, mul2, nbase2);
-        const float2 e = make_float2(fast_exp2(arg.x), fast_exp2(arg.y));
-        sum4[(c >> 1) & 3] = __fadd2_rn(sum4[(c >> 1) & 3], e);
-        pk[c / 2] = pack_bf16x2(e.x, e.y);
-      }
-      tmem_st16(s_addr + h * 32 + ch * 16, pk);
-    }
-    const float2 s01 = __fadd2_rn(sum4[0], sum4[1]), s23 = __fadd2_rn(sum4[2], sum4[3]);
-    const float2 s03 = __fadd2_rn(s01, s23);
-    sum = s03.x + s03.y;
-  }
-  l_half = l_half * alpha + sum;
+  for (int a = 0; a < 4; ++a) sum4[a] = make_float2(0.f, 0.f);
+  exp32<false>(s_addr, v, mul, base, sum4, nullptr);
+  exp32<false>(s_addr + 16, v + 32, mul, base, sum4, nullptr);
+  l_half = l_half * alpha + sum_of(sum4);
   m_run = m_new;
   return alpha;
+}
+
+// softmax_half_based: the base is the row's m_run as it is (any base within
+// 2^kWindowLog2 below the maximum gives the same result after the final
+// normalisation: fp32 and bf16 have the exponents for it), so the halves
+// exchange nothing and no maximum is waited for.  Returns false when a score
+// of this thread lies above the window.
+__device__ __forceinline__ bool softmax_half_based(uint32_t s_addr, int lo, int hi, float sl2,
+                                                   float m_run, float &l_half) {
+  using namespace sm100;
+  const float NEG_INF = -__int_as_float(0x7f800000);
+  if (__all_sync(0xffffffffu, hi <= lo)) {  // no row of the warp sees a key of the half
+    uint32_t z[32];
+#pragma unroll
+    for (int c = 0; c < 32; ++c) z[c] = 0u;
+    tmem_st32(s_addr, z);
+    return true;
+  }
+  const bool raw = sl2 > 0.f;
+  const bool plain = __all_sync(0xffffffffu, raw && lo <= 0 && hi >= 64);
+  const float mul = raw ? sl2 : 1.f, base = m_run == NEG_INF ? 0.f : m_run;
+  uint32_t v[64];
+  float2 sum4[4];
+  float mx4[4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    sum4[a] = make_float2(0.f, 0.f);
+    mx4[a] = NEG_INF;
+  }
+  tmem_ld32(s_addr, v);
+  tmem_ld_wait32(v);
+  tmem_ld32(s_addr + 32, v + 32);
+  if (!plain) mask32(v, lo, hi, !raw, sl2);
+  exp32<true>(s_addr, v, mul, base, sum4, mx4);
+  tmem_ld_wait32(v + 32);
+  if (!plain) mask32(v + 32, lo - 32, hi - 32, !raw, sl2);
+  exp32<true>(s_addr + 16, v + 32, mul, base, sum4, mx4);
+  l_half += sum_of(sum4);
+  // (not >, so that a NaN leaves the window too)
+  return fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * mul <= base + kWindowLog2;
 }
 
 // ------------------------------------------------------------------ host --

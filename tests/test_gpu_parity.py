@@ -454,3 +454,34 @@ def test_ratio_that_does_not_divide_the_tile(hpd, hq, hkv, m, D):
         out, lse, err = run_gpu(hpd, W.page_the_prefix(inp, seed=95) if paged else inp)
         assert err == 0
         compare(inp, out, lse, ref_out, ref_lse)
+
+
+@pytest.mark.parametrize("hq,hkv,D,n", [(16, 2, 128, 40), (8, 2, 64, 3)])
+def test_scores_that_leave_the_window_of_their_base(hpd, hq, hkv, D, n):
+    # A row's exponentials are taken against the maximum of its first block
+    # until a score exceeds it by 2^64; the unit then runs once more.  Keys far
+    # longer than the first block's, in the prefix (from key 200 of page 0, the
+    # last key of page 1) and among private keys, make scores of some hundreds;
+    # page 2 stays inside.  The oracle's rows are then one key's value almost
+    # everywhere, so an error of the bf16 weights does not average out: a
+    # weight near 1/2 rounded to bf16 (2^-9 relative) times a value of up to 4
+    # in the bound of 1e-2; the scores' own fp32 rounding (2^-24 * 128 terms of
+    # up to 100) is below the lse's 1e-3.
+    inp = W.build_inputs([700, 257, 300], [n, 5, 2], [(13 * b) % 300 for b in range(n + 7)], 4, hq,
+                         hkv, D, seed=53)
+    k = W.bf16_bits_to_f32(inp.prefix_k)
+    k[200:700] *= 120.0
+    k[700 + 256] *= 150.0
+    inp.prefix_k = W.f32_to_bf16_bits(k)
+    kc = W.bf16_bits_to_f32(inp.k_cache)
+    kc[inp.page_table[n + 1, 0]] *= 130.0
+    inp.k_cache = W.f32_to_bf16_bits(kc)
+    ref_out, ref_lse = oracle.branch_attn(inp)
+    assert np.max(ref_lse) > 64.0 * np.log(2.0)
+    d = hpd.DeviceInputs.from_host(inp)
+    op = hpd.BranchAttn(d)
+    for _ in range(2):  # the second call finds every counter as the first did
+        out, lse = op()
+        torch.cuda.synchronize()
+        assert op.errors() == 0
+        compare(inp, out.float().cpu().numpy(), lse.cpu().numpy(), ref_out, ref_lse)
