@@ -568,121 +568,113 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Shared-memory descriptors: a slot / stage / k-step offset only adds
     // (offset >> 4) to the start-address field (bits 0-13), which cannot
     // carry: every address stays below 256 KB.
+    // V is MN-major (D contiguous): 64-column swizzle atoms kChunkBytes apart
+    // along N (leading byte offset), 8-key groups 1024 bytes apart along K
+    // (stride byte offset).
     const uint64_t dk0 = smem_desc_sw128(sbase + L::kK, 16, 1024);
-    // S[col] = Q (TMEM slot qs) K^T of global block jg: A from TMEM, 16
-    // dimensions (8 columns) per MMA; B = K, K-major in shared memory
-    // (one lane, elected once per group, issues the group's MMAs and commits)
-    const bool issuer = elect_one();
-    auto issue_qk = [&](int qs, int sk, uint32_t col) {
-      const uint64_t kd = dk0 + ((sk * L::kTileBytes) >> 4);
-      if (issuer) {
-#pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-          const uint32_t off = ((kk >> 2) * L::kChunkBytes + (kk & 3) * 32) >> 4;
-          mma_ts_one(tmem + col, tmem + L::col_q(qs) + kk * 8, kd + off, idesc_qk, kk > 0);
-        }
-      }
-      __syncwarp();
-    };
-    auto commit = [&](uint64_t &b) {
-      if (issuer) mma_commit_one(bar(b));
-      __syncwarp();
-    };
-    // O (+)= P V of global block jg, P in TMEM at column pcol: one
-    // N = D MMA per 16 keys.  V is MN-major (D contiguous): 64-column swizzle
-    // atoms kChunkBytes apart along N (leading byte offset), 8-key groups
-    // 1024 bytes apart along K (stride byte offset).
     const uint64_t dv0 = smem_desc_sw128(sbase + L::kV, L::kChunkBytes, 1024);
-    auto issue_pv = [&](int jg, bool first, uint32_t pcol) {
-      const uint64_t vd = dv0 + (((jg % L::kVStages) * L::kTileBytes) >> 4);
-      if (issuer) {
-#pragma unroll
-        for (int kk = 0; kk < kBlk / 16; ++kk)
-          mma_ts_one(tmem + L::kColO, tmem + pcol + kk * 8 + (kk >= 4 ? 32 : 0), vd + ((kk * 16 * 128) >> 4), idesc_pv,
-                     (!first || kk > 0) ? 1u : 0u);
+    const bool issuer = elect_one();
+    // Ring positions and S buffers advance by counting: the warp's own
+    // instructions between the MMAs it issues are time the tensor cores idle.
+    uint32_t sk = 0, pk = 0;  // next K ring entry: stage, phase
+    uint32_t sv = 0, pv = 0;  // next V ring entry
+    uint32_t sq = 0;          // S buffer of the next Q K^T
+    uint32_t so = 0, po = 0;  // S buffer (and P) of the next P V, its phase
+    auto advance = [](uint32_t &st, uint32_t &ph, uint32_t n) {
+      if (++st == n) {
+        st = 0;
+        ph ^= 1u;
       }
-      __syncwarp();
     };
-    auto wait = [&](uint64_t &b, int parity) {
-      if (!wait_bar(b, parity)) return false;
-      tc_fence_after();
-      return true;
-    };
-    // The P V of a block is issued after the Q K^T of the next block (QK(b),
-    // PV(b-1)), across unit boundaries too.
-    struct Pending {
-      int jg, unit;
-      bool first, last;
-    };
-    Pending pend{0, 0, false, false};
-    bool has_pend = false;
-    // V of block x.jg and K of block jn (the next Q K^T) are tested while
-    // the warp waits for P of block x.jg, so that their shared-memory round
-    // trips overlap; only phases not yet complete are waited for again.
-    // k_next: K of block jn has landed.
-    // (jn: ring entry of the next K block, or -1 when the next entry is a Q)
-    auto do_pv = [&](const Pending &x, int jn, bool &k_next) -> bool {
-      const int s = x.jg & 1, sv = x.jg % L::kVStages;
-      const int kb = jn >= 0 ? bar(sh.k_full[jn % L::kKStages]) : bar(sh.v_full[sv]);
-      const int kp = jn >= 0 ? (jn / L::kKStages) & 1 : (x.jg / L::kVStages) & 1;
-      uint32_t r = mbar_try_test2(bar(sh.p_full[s]), (x.jg >> 1) & 1, bar(sh.v_full[sv]),
-                                  (x.jg / L::kVStages) & 1, kb, kp);
-      r = __shfl_sync(0xffffffffu, r, 0);
-      k_next = jn >= 0 && (r & 4u) != 0;
-      if (!(r & 1u) && !wait_bar(sh.p_full[s], (x.jg >> 1) & 1)) return false;
-      if (!(r & 2u) && !wait_bar(sh.v_full[sv], (x.jg / L::kVStages) & 1)) return false;
-      tc_fence_after();
-      // O last held unit x.unit - 1, whose epilogue must have read it
-      if (x.first && x.unit >= 1 && !wait(sh.o_empty, (x.unit - 1) & 1)) return false;
-      issue_pv(x.jg, x.first, L::col_s(s));
-      commit(sh.pv_done);
-      commit(sh.v_empty[sv]);
-      if (x.last) commit(sh.o_full);
-      return true;
-    };
-    int jbase = 0;
-    bool ok = true, k_ready = false;
+    bool pend = false;               // a block whose P V is still to come
+    bool pend_first = false, pend_last = false;  // of its unit,
+    int pend_unit = 0;                           // which is this one
+    bool ok = true, k_ready = false;  // (k_ready: the next K entry was seen full)
     for (int k = 0; ok; ++k) {
       const int slot = k & 1;
-      // no next unit yet: the scheduler may be waiting for this one's end
-      if (has_pend && !__all_sync(0xffffffffu, mbar_test_wait(bar(sh.meta_full[slot]), (k >> 1) & 1))) {
-        if (!(ok = do_pv(pend, -1, k_ready))) break;
-        has_pend = false;
-      }
-      if (!(ok = wait(sh.meta_full[slot], (k >> 1) & 1))) break;
+      if (!(ok = wait_bar(sh.meta_full[slot], (k >> 1) & 1))) break;
       const bool valid = meta[slot].valid != 0;
       const int nb = meta[slot].n_blocks;
       __syncwarp();
       if (!valid) break;
       if (lane == 0) mbar_arrive(bar(sh.meta_empty[slot]));
-      // the unit's Q: from its K-ring entry into TMEM slot qs (the copy runs
-      // in order with the MMAs: unit k - 2's Q K^T are done with the slot)
-      const int qs = k & 1, qe = jbase + k, sq = qe % L::kKStages;
-      if (!(ok = wait(sh.k_full[sq], (qe / L::kKStages) & 1))) break;
+      // the unit's Q: from its K-ring entry into TMEM slot k & 1 (the copy
+      // runs in order with the MMAs: unit k - 2's Q K^T are done with it)
+      if (!(ok = wait_bar(sh.k_full[sk], pk))) break;
+      tc_fence_after();
       if (issuer) {
-        const uint64_t qd = dk0 + ((sq * L::kTileBytes) >> 4);
+        const uint64_t qd = dk0 + ((sk * L::kTileBytes) >> 4);
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk)
-          tmem_cp_128x256b(tmem + L::col_q(qs) + kk * 8,
+          tmem_cp_128x256b(tmem + L::col_q(slot) + kk * 8,
                            qd + (((kk >> 2) * L::kChunkBytes + (kk & 3) * 32) >> 4));
+        mma_commit_one(bar(sh.k_empty[sk]));
       }
       __syncwarp();
-      commit(sh.k_empty[sq]);
+      advance(sk, pk, L::kKStages);
       k_ready = false;
-      for (int j = 0; j < nb; ++j) {
-        const int jg = jbase + j, s = jg & 1, ke = jg + k + 1, sk = ke % L::kKStages;
-        if (!k_ready && !(ok = wait(sh.k_full[sk], (ke / L::kKStages) & 1))) break;
-        issue_qk(qs, sk, L::col_s(s));
-        commit(sh.s_full[s]);
-        commit(sh.k_empty[sk]);
-        k_ready = false;
-        if (has_pend && !(ok = do_pv(pend, j + 1 < nb ? ke + 1 : -1, k_ready))) break;
-        pend = Pending{jg, k, j == 0, j == nb - 1};
-        has_pend = true;
+      // QK(j), PV(j - 1), across unit boundaries too, unless no next unit is
+      // there yet when this one ends (the scheduler may be waiting for that
+      // end): then its last P V comes alone
+      for (int j = 0;
+           j < nb || (j == nb && pend &&
+                      !__all_sync(0xffffffffu, mbar_test_wait(bar(sh.meta_full[slot ^ 1]),
+                                                              ((k + 1) >> 1) & 1)));
+           ++j) {
+        if (j < nb) {
+          if (!k_ready && !(ok = wait_bar(sh.k_full[sk], pk))) break;
+          if (issuer) {
+            // S = Q K^T: A from TMEM, 16 dimensions (8 columns) per MMA; K is
+            // K-major in shared memory
+            const uint64_t kd = dk0 + ((sk * L::kTileBytes) >> 4);
+            const uint32_t col = tmem + (sq ? L::col_s(1) : L::col_s(0));
+#pragma unroll
+            for (int kk = 0; kk < D / 16; ++kk)
+              mma_ts_one(col, tmem + L::col_q(slot) + kk * 8,
+                         kd + (((kk >> 2) * L::kChunkBytes + (kk & 3) * 32) >> 4), idesc_qk, kk > 0);
+            mma_commit_one(bar(sh.s_full[sq]));
+            mma_commit_one(bar(sh.k_empty[sk]));
+          }
+          advance(sk, pk, L::kKStages);
+          sq ^= 1u;
+          k_ready = false;
+        }
+        if (pend) {
+          // V of the block and the next K are tested while the warp waits for
+          // P, so that their shared-memory round trips overlap; only phases
+          // not yet complete are waited for again
+          uint32_t r = mbar_try_test2(bar(sh.p_full[so]), po, bar(sh.v_full[sv]), pv,
+                                      bar(sh.k_full[sk]), pk);
+          r = __shfl_sync(0xffffffffu, r, 0);
+          // (the entry after a unit's last block is the next unit's Q)
+          k_ready = j + 1 < nb && (r & 4u) != 0;
+          if (!(r & 1u) && !(ok = wait_bar(sh.p_full[so], po))) break;
+          if (!(r & 2u) && !(ok = wait_bar(sh.v_full[sv], pv))) break;
+          // O last held the unit before, whose epilogue must have read it
+          if (pend_first && pend_unit >= 1 && !(ok = wait_bar(sh.o_empty, (pend_unit - 1) & 1))) break;
+          tc_fence_after();
+          if (issuer) {
+            // O (+)= P V: 16 keys per MMA, P in the S buffer (half h of the
+            // keys at column 64 h)
+            const uint64_t vd = dv0 + ((sv * L::kTileBytes) >> 4);
+            const uint32_t col = tmem + (so ? L::col_s(1) : L::col_s(0));
+#pragma unroll
+            for (int kk = 0; kk < kBlk / 16; ++kk)
+              mma_ts_one(tmem + L::kColO, col + kk * 8 + (kk >= 4 ? 32 : 0),
+                         vd + ((kk * 16 * 128) >> 4), idesc_pv, (!pend_first || kk > 0) ? 1u : 0u);
+            mma_commit_one(bar(sh.pv_done));
+            mma_commit_one(bar(sh.v_empty[sv]));
+            if (pend_last) mma_commit_one(bar(sh.o_full));
+          }
+          advance(sv, pv, L::kVStages);
+          advance(so, po, 2);
+        }
+        pend = j < nb;
+        pend_first = j == 0;
+        pend_last = j == nb - 1;
+        pend_unit = k;
       }
-      jbase += nb;
     }
-    if (ok && has_pend) ok = do_pv(pend, -1, k_ready);
     if (!ok && lane == 0) set_abort(sh, p.err);
   } else {
     // --------------------------------------------------------- softmax --
@@ -700,6 +692,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool unit;  // false: no unit left
       bool valid, exact;
       int g, split, nb, blk_lo, nP, lim_p, ps, last;
+      int n_plain;  // leading prefix blocks of which every row of the warp sees all keys
       size_t pair;
     };
     // Reads unit k's metadata (slot k & 1) and releases the slot (the unit's
@@ -720,7 +713,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         R.exact = M.exact != 0;
         const int rt = p.div_G(r_in), token = M.tok0 + rt;
         const int bl = R.valid ? p.div_m(token) - M.b_lo : 0;
-        R.lim_p = R.valid ? M.fork[bl] : 0;
+        // (rows that are no query count as seeing the whole prefix, so that
+        // their warp needs no masks there; their results are not stored)
+        R.lim_p = R.valid ? M.fork[bl] : R.nP * kBlk;
+        R.n_plain = sl2 > 0.f ? __reduce_min_sync(0xffffffffu, R.lim_p) / kBlk : 0;
         R.ps = R.valid ? M.page_start[bl] : 0;
         R.last = R.valid ? M.blen[bl] - m + (token - (M.b_lo + bl) * m) : -1;
         R.pair = static_cast<size_t>(token) * p.H_q + R.g * G + r_in - rt * G;
@@ -737,24 +733,28 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!(ok = begin_unit(k, cur)) || !cur.unit) break;
       float m_run = NEG_INF, l_half = 0.f;
       bool inside = true;  // the scores stay in the window of their base
+      // A row's base is the maximum of the first block it sees keys of; both
+      // halves come to the same answer when that is, and take that block's
+      // maximum together (exact: every block's).
+      bool based = false;  // every row of the warp has its base
       for (int j = 0; j < cur.nb; ++j) {
         const int jg = jbase + j;
         const int si = jg & 1;
         const int jb = cur.blk_lo + j;
-        int lo, hi;
-        if (jb < cur.nP) {
-          lo = 0;
-          hi = cur.lim_p - jb * kBlk;
-        } else {
-          const int off = (cur.ps - (jb - cur.nP) * kPagesPerBlock) * kPage;  // column of own key 0
-          lo = max(0, off);
-          hi = min(kBlk, off + cur.last + 1);
+        const bool plain = jb < cur.n_plain;
+        int lo = 0, hi = kBlk;
+        bool find_max = cur.exact || !based;
+        if (!plain) {
+          if (jb < cur.nP) {
+            hi = min(cur.lim_p - jb * kBlk, kBlk);
+          } else {
+            const int off = (cur.ps - (jb - cur.nP) * kPagesPerBlock) * kPage;  // column of own key 0
+            lo = max(0, off);
+            hi = min(kBlk, off + cur.last + 1);
+          }
+          if (!cur.exact && !based)
+            find_max = __any_sync(0xffffffffu, cur.valid && m_run == NEG_INF && hi > lo);
         }
-        // A row's base is the maximum of the first block it sees keys of;
-        // both halves come to the same answer here, and take that block's
-        // maximum together.  (exact: every block's.)
-        const bool find_max =
-            cur.exact || __any_sync(0xffffffffu, m_run == NEG_INF && min(hi, kBlk) > lo);
         // warp-uniform outcome: the tcgen05.ld / st below are warp-collective
         if (!(ok = wait_bar(sh.s_full[si], (jg >> 1) & 1))) break;
         tc_fence_after();
@@ -762,7 +762,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         bool rescale = false;
         float alpha = 1.f;
         if (!find_max) {
-          inside &= tc::softmax_half_based(s_addr, lo - h * 64, hi - h * 64, sl2, m_run, l_half);
+          inside &= tc::softmax_half_based(s_addr, plain, lo - h * 64, hi - h * 64, sl2, m_run, l_half);
         } else {
           const int par = jg & 1;
           bool xok = true;
@@ -775,6 +775,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           alpha = tc::softmax_half_max(s_addr, lo - h * 64, hi - h * 64, sl2, m_run, l_half, xchg);
           if (!(ok = __all_sync(0xffffffffu, xok))) break;
           rescale = __any_sync(0xffffffffu, j > 0 && alpha != 1.f);
+          based = __all_sync(0xffffffffu, !cur.valid || m_run != NEG_INF);
         }
         // Before O may be rescaled, the P V MMA of block jg-1 must have
         // landed: a warp that rescales waits for it.  Warps skip the wait
@@ -785,11 +786,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (rescale) {
           if (!(ok = wait_bar(sh.pv_done, (jg - 1) & 1))) break;
           tc_fence_after();
-#pragma unroll
+#pragma unroll 1
           for (int c = 0; c < D / 2; c += 32) {
             uint32_t o[32];
             tmem_ld32(t_lane + o_col + c, o);
-            tmem_ld_wait();
+            tmem_ld_wait32(o);
 #pragma unroll
             for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
             tmem_st32(t_lane + o_col + c, o);
@@ -819,11 +820,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float lse = l_run > 0.f ? (m_run + __log2f(l_run)) * kLn2 : NEG_INF;
       const bool final_out = p.S_p == 1;
       const size_t slot_pair = static_cast<size_t>(cur.split) * p.rows_total * p.H_q + cur.pair;
-#pragma unroll
+#pragma unroll 1
       for (int c = 0; c < D / 2; c += 32) {
         uint32_t o[32];
         tmem_ld32(t_lane + o_col + c, o);
-        tmem_ld_wait();
+        tmem_ld_wait32(o);
         if (!cur.valid) continue;
         const int dc = h * (D / 2) + c;  // output column
         // 32-byte stores: each fills a whole sector of its row

@@ -117,13 +117,14 @@ __device__ __forceinline__ float softmax_half_max(uint32_t s_addr, int lo, int h
 // softmax_half_based: the base is the row's m_run as it is (any base within
 // 2^kWindowLog2 below the maximum gives the same result after the final
 // normalisation: fp32 and bf16 have the exponents for it), so the halves
-// exchange nothing and no maximum is waited for.  Returns false when a score
-// of this thread lies above the window.
-__device__ __forceinline__ bool softmax_half_based(uint32_t s_addr, int lo, int hi, float sl2,
-                                                   float m_run, float &l_half) {
+// exchange nothing and no maximum is waited for.  plain: every row of the warp sees
+// every key, and the scale is positive.  Returns false when a score of this
+// thread lies above the window.
+__device__ __forceinline__ bool softmax_half_based(uint32_t s_addr, bool plain, int lo, int hi,
+                                                   float sl2, float m_run, float &l_half) {
   using namespace sm100;
   const float NEG_INF = -__int_as_float(0x7f800000);
-  if (__all_sync(0xffffffffu, hi <= lo)) {  // no row of the warp sees a key of the half
+  if (!plain && __all_sync(0xffffffffu, hi <= max(lo, 0))) {  // no row of the warp sees a key of the half
     uint32_t z[32];
 #pragma unroll
     for (int c = 0; c < 32; ++c) z[c] = 0u;
@@ -131,7 +132,6 @@ __device__ __forceinline__ bool softmax_half_based(uint32_t s_addr, int lo, int 
     return true;
   }
   const bool raw = sl2 > 0.f;
-  const bool plain = __all_sync(0xffffffffu, raw && lo <= 0 && hi >= 64);
   const float mul = raw ? sl2 : 1.f, base = m_run == NEG_INF ? 0.f : m_run;
   uint32_t v[64];
   float2 sum4[4];
