@@ -36,16 +36,17 @@
 //               blocks, warp 11 its V blocks, each into a three-stage ring
 //               (128-byte swizzle); a K stage is refilled as soon as its Q
 //               K^T (or Q copy) is done, whatever the V ring waits for.
-//   warp 1      TMEM owner and MMA issuer: copies each unit's Q tile from
-//               its K stage into TMEM (tcgen05.cp, double buffered by unit),
-//               then one global sequence of blocks across units, in the
-//               order QK(b), PV(b-1):
+//   warps 1, 12 MMA issuers (warp 1 owns TMEM).  Warp 1 copies each unit's
+//               Q tile from its K stage into TMEM (tcgen05.cp, double
+//               buffered by unit) and issues
 //                 S = Q K^T   Q read from TMEM, K from shared memory; S into
 //                             TMEM (fp32, double buffered by block)
+//               and warp 12
 //                 O += P V    P read from TMEM (bf16, written over S), V from
 //                             shared memory; O accumulated in TMEM
 //               With both A operands in TMEM, shared memory serves only K,
-//               V and their TMA writes (its bandwidth is the scarce port).
+//               V and their TMA writes.  Each warp's waits and bookkeeping
+//               pass while the other's MMAs run.
 //   warps 2..9  softmax: two warpgroups, each owning half of every block's
 //               128 key columns and half of O's columns; thread t of warp w
 //               owns TMEM lane 32*(w%4)+t, i.e. one query row.  The two
@@ -89,9 +90,10 @@ constexpr int kPagesPerBlock = kBlk / kPage;
 constexpr int kSoftmaxWarps = 8;
 constexpr int kSchedWarp = 2 + kSoftmaxWarps;
 constexpr int kVWarp = kSchedWarp + 1;
-constexpr int kThreads = 32 * (kVWarp + 1);
-// consumers of a metadata slot: two producers, MMA issuer, softmax warps
-constexpr uint32_t kMetaConsumers = 3 + kSoftmaxWarps;
+constexpr int kPvWarp = kVWarp + 1;
+constexpr int kThreads = 32 * (kPvWarp + 1);
+// consumers of a metadata slot: two producers, two MMA issuers, softmax warps
+constexpr uint32_t kMetaConsumers = 4 + kSoftmaxWarps;
 constexpr int kMaxRing = 3;  // largest K / V ring
 
 // Metadata of one unit, written by the scheduler warp.
@@ -139,10 +141,11 @@ struct __align__(8) TcShared {
   uint64_t meta_full[2], meta_empty[2];
   uint64_t k_full[kMaxRing], v_full[kMaxRing];
   uint64_t k_empty[kMaxRing], v_empty[kMaxRing];
-  uint64_t s_full[2], p_full[2];  // per S buffer
-  uint64_t pv_done;
+  // per S buffer: scores written; P written; P V done (the buffer is free and
+  // O holds the block)
+  uint64_t s_full[2], p_full[2], s_free[2];
   uint64_t o_full, o_empty;
-  uint64_t mma_done;
+  uint64_t mma_done[2];
   uint32_t tmem_base;
   int abort;
   // the two column halves of a row exchange their partial row max (double
@@ -248,11 +251,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(bar(sh.meta_empty[s]), kMetaConsumers);
       mbar_init(bar(sh.s_full[s]), 1);
       mbar_init(bar(sh.p_full[s]), kSoftmaxWarps);
+      mbar_init(bar(sh.s_free[s]), 1);
     }
-    mbar_init(bar(sh.pv_done), 1);
     mbar_init(bar(sh.o_full), 1);
     mbar_init(bar(sh.o_empty), kSoftmaxWarps);
-    mbar_init(bar(sh.mma_done), 1);
+    mbar_init(bar(sh.mma_done[0]), 1);
+    mbar_init(bar(sh.mma_done[1]), 1);
     fence_mbar_init();
   }
   if (tid < 16) (&sh.xseq[0][0][0])[tid] = 0;
@@ -560,36 +564,20 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int e = max(0, issued - L::kKStages); e < issued; ++e)
       mbar_wait(bar(full[e % L::kKStages]), (e / L::kKStages) & 1);
   } else if (warp == 1) {
-    // ------------------------------------------------------ MMA issuer --
+    // ---------------------------------------------------- Q K^T issuer --
     // The whole warp runs this loop with warp-uniform values; one elected
-    // lane issues each MMA / commit (see sm100.cuh).
+    // lane issues each group of MMAs and its commits (see sm100.cuh).  Stages
+    // and phases advance by counting: the warp's own instructions between the
+    // MMAs are time the tensor cores may idle.
     constexpr uint32_t idesc_qk = idesc_bf16_f32(kRows, kBlk, false);
-    constexpr uint32_t idesc_pv = idesc_bf16_f32(kRows, D, true);
-    // Shared-memory descriptors: a slot / stage / k-step offset only adds
-    // (offset >> 4) to the start-address field (bits 0-13), which cannot
-    // carry: every address stays below 256 KB.
-    // V is MN-major (D contiguous): 64-column swizzle atoms kChunkBytes apart
-    // along N (leading byte offset), 8-key groups 1024 bytes apart along K
-    // (stride byte offset).
+    // Shared-memory descriptors: a stage / k-step offset only adds (offset >>
+    // 4) to the start-address field (bits 0-13), which cannot carry: every
+    // address stays below 256 KB.
     const uint64_t dk0 = smem_desc_sw128(sbase + L::kK, 16, 1024);
-    const uint64_t dv0 = smem_desc_sw128(sbase + L::kV, L::kChunkBytes, 1024);
     const bool issuer = elect_one();
-    // Ring positions and S buffers advance by counting: the warp's own
-    // instructions between the MMAs it issues are time the tensor cores idle.
-    uint32_t sk = 0, pk = 0;  // next K ring entry: stage, phase
-    uint32_t sv = 0, pv = 0;  // next V ring entry
-    uint32_t sq = 0;          // S buffer of the next Q K^T
-    uint32_t so = 0, po = 0;  // S buffer (and P) of the next P V, its phase
-    auto advance = [](uint32_t &st, uint32_t &ph, uint32_t n) {
-      if (++st == n) {
-        st = 0;
-        ph ^= 1u;
-      }
-    };
-    bool pend = false;               // a block whose P V is still to come
-    bool pend_first = false, pend_last = false;  // of its unit,
-    int pend_unit = 0;                           // which is this one
-    bool ok = true, k_ready = false;  // (k_ready: the next K entry was seen full)
+    uint32_t sk = 0, pk = 0;  // K ring: stage, phase
+    int jg = 0;               // blocks issued
+    bool ok = true;
     for (int k = 0; ok; ++k) {
       const int slot = k & 1;
       if (!(ok = wait_bar(sh.meta_full[slot], (k >> 1) & 1))) break;
@@ -598,81 +586,84 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (!valid) break;
       if (lane == 0) mbar_arrive(bar(sh.meta_empty[slot]));
-      // the unit's Q: from its K-ring entry into TMEM slot k & 1 (the copy
-      // runs in order with the MMAs: unit k - 2's Q K^T are done with it)
-      if (!(ok = wait_bar(sh.k_full[sk], pk))) break;
-      tc_fence_after();
-      if (issuer) {
-        const uint64_t qd = dk0 + ((sk * L::kTileBytes) >> 4);
+      // entry -1 of the unit: its Q, copied into TMEM slot k & 1 (in order
+      // with the MMAs: unit k - 2's Q K^T are done with the slot)
+      for (int j = -1; j < nb; ++j) {
+        if (!(ok = wait_bar(sh.k_full[sk], pk))) break;
+        // the S buffer is free once P V of the block before last has read P
+        if (j >= 0 && jg >= 2 && !(ok = wait_bar(sh.s_free[jg & 1], ((jg >> 1) - 1) & 1))) break;
+        tc_fence_after();
+        if (issuer) {
+          const uint64_t kd = dk0 + ((sk * L::kTileBytes) >> 4);
+          if (j < 0) {
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk)
-          tmem_cp_128x256b(tmem + L::col_q(slot) + kk * 8,
-                           qd + (((kk >> 2) * L::kChunkBytes + (kk & 3) * 32) >> 4));
-        mma_commit_one(bar(sh.k_empty[sk]));
-      }
-      __syncwarp();
-      advance(sk, pk, L::kKStages);
-      k_ready = false;
-      // QK(j), PV(j - 1), across unit boundaries too, unless no next unit is
-      // there yet when this one ends (the scheduler may be waiting for that
-      // end): then its last P V comes alone
-      for (int j = 0;
-           j < nb || (j == nb && pend &&
-                      !__all_sync(0xffffffffu, mbar_test_wait(bar(sh.meta_full[slot ^ 1]),
-                                                              ((k + 1) >> 1) & 1)));
-           ++j) {
-        if (j < nb) {
-          if (!k_ready && !(ok = wait_bar(sh.k_full[sk], pk))) break;
-          if (issuer) {
-            // S = Q K^T: A from TMEM, 16 dimensions (8 columns) per MMA; K is
-            // K-major in shared memory
-            const uint64_t kd = dk0 + ((sk * L::kTileBytes) >> 4);
-            const uint32_t col = tmem + (sq ? L::col_s(1) : L::col_s(0));
+            for (int kk = 0; kk < D / 16; ++kk)
+              tmem_cp_128x256b(tmem + L::col_q(slot) + kk * 8,
+                               kd + (((kk >> 2) * L::kChunkBytes + (kk & 3) * 32) >> 4));
+          } else {
+            // A from TMEM, 16 dimensions (8 columns) per MMA; K is K-major
+            const uint32_t col = tmem + L::col_s(jg & 1);
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk)
               mma_ts_one(col, tmem + L::col_q(slot) + kk * 8,
                          kd + (((kk >> 2) * L::kChunkBytes + (kk & 3) * 32) >> 4), idesc_qk, kk > 0);
-            mma_commit_one(bar(sh.s_full[sq]));
-            mma_commit_one(bar(sh.k_empty[sk]));
+            mma_commit_one(bar(sh.s_full[jg & 1]));
           }
-          advance(sk, pk, L::kKStages);
-          sq ^= 1u;
-          k_ready = false;
+          mma_commit_one(bar(sh.k_empty[sk]));
         }
-        if (pend) {
-          // V of the block and the next K are tested while the warp waits for
-          // P, so that their shared-memory round trips overlap; only phases
-          // not yet complete are waited for again
-          uint32_t r = mbar_try_test2(bar(sh.p_full[so]), po, bar(sh.v_full[sv]), pv,
-                                      bar(sh.k_full[sk]), pk);
-          r = __shfl_sync(0xffffffffu, r, 0);
-          // (the entry after a unit's last block is the next unit's Q)
-          k_ready = j + 1 < nb && (r & 4u) != 0;
-          if (!(r & 1u) && !(ok = wait_bar(sh.p_full[so], po))) break;
-          if (!(r & 2u) && !(ok = wait_bar(sh.v_full[sv], pv))) break;
-          // O last held the unit before, whose epilogue must have read it
-          if (pend_first && pend_unit >= 1 && !(ok = wait_bar(sh.o_empty, (pend_unit - 1) & 1))) break;
-          tc_fence_after();
-          if (issuer) {
-            // O (+)= P V: 16 keys per MMA, P in the S buffer (half h of the
-            // keys at column 64 h)
-            const uint64_t vd = dv0 + ((sv * L::kTileBytes) >> 4);
-            const uint32_t col = tmem + (so ? L::col_s(1) : L::col_s(0));
+        __syncwarp();
+        if (++sk == L::kKStages) {
+          sk = 0;
+          pk ^= 1u;
+        }
+        jg += j >= 0;
+      }
+    }
+    if (!ok && lane == 0) set_abort(sh, p.err);
+  } else if (warp == kPvWarp) {
+    // ------------------------------------------------------ P V issuer --
+    constexpr uint32_t idesc_pv = idesc_bf16_f32(kRows, D, true);
+    // V is MN-major (D contiguous): 64-column swizzle atoms kChunkBytes apart
+    // along N (leading byte offset), 8-key groups 1024 bytes apart along K
+    // (stride byte offset).
+    const uint64_t dv0 = smem_desc_sw128(sbase + L::kV, L::kChunkBytes, 1024);
+    const bool issuer = elect_one();
+    uint32_t sv = 0, pv = 0;  // V ring: stage, phase
+    int jg = 0;               // blocks issued
+    bool ok = true;
+    for (int k = 0; ok; ++k) {
+      const int slot = k & 1;
+      if (!(ok = wait_bar(sh.meta_full[slot], (k >> 1) & 1))) break;
+      const bool valid = meta[slot].valid != 0;
+      const int nb = meta[slot].n_blocks;
+      __syncwarp();
+      if (!valid) break;
+      if (lane == 0) mbar_arrive(bar(sh.meta_empty[slot]));
+      // O last held the unit before, whose epilogue must have read it
+      if (k >= 1 && !(ok = wait_bar(sh.o_empty, (k - 1) & 1))) break;
+      for (int j = 0; j < nb; ++j) {
+        if (!(ok = wait_bar(sh.v_full[sv], pv))) break;
+        if (!(ok = wait_bar(sh.p_full[jg & 1], (jg >> 1) & 1))) break;
+        tc_fence_after();
+        if (issuer) {
+          // O (+)= P V: 16 keys per MMA, P in the S buffer (half h of the keys
+          // at column 64 h)
+          const uint64_t vd = dv0 + ((sv * L::kTileBytes) >> 4);
+          const uint32_t col = tmem + L::col_s(jg & 1);
 #pragma unroll
-            for (int kk = 0; kk < kBlk / 16; ++kk)
-              mma_ts_one(tmem + L::kColO, col + kk * 8 + (kk >= 4 ? 32 : 0),
-                         vd + ((kk * 16 * 128) >> 4), idesc_pv, (!pend_first || kk > 0) ? 1u : 0u);
-            mma_commit_one(bar(sh.pv_done));
-            mma_commit_one(bar(sh.v_empty[sv]));
-            if (pend_last) mma_commit_one(bar(sh.o_full));
-          }
-          advance(sv, pv, L::kVStages);
-          advance(so, po, 2);
+          for (int kk = 0; kk < kBlk / 16; ++kk)
+            mma_ts_one(tmem + L::kColO, col + kk * 8 + (kk >= 4 ? 32 : 0),
+                       vd + ((kk * 16 * 128) >> 4), idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
+          mma_commit_one(bar(sh.s_free[jg & 1]));
+          mma_commit_one(bar(sh.v_empty[sv]));
+          if (j == nb - 1) mma_commit_one(bar(sh.o_full));
         }
-        pend = j < nb;
-        pend_first = j == 0;
-        pend_last = j == nb - 1;
-        pend_unit = k;
+        __syncwarp();
+        if (++sv == L::kVStages) {
+          sv = 0;
+          pv ^= 1u;
+        }
+        ++jg;
       }
     }
     if (!ok && lane == 0) set_abort(sh, p.err);
@@ -778,13 +769,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           based = __all_sync(0xffffffffu, !cur.valid || m_run != NEG_INF);
         }
         // Before O may be rescaled, the P V MMA of block jg-1 must have
-        // landed: a warp that rescales waits for it.  Warps skip the wait
-        // when they do not rescale, yet the parity test stays exact: Q K^T
-        // (jg) was issued after P V (jg-2), so the S commit awaited above
-        // implies P V (jg-2) has completed, and P V (jg) needs this block's
-        // P; the barrier is in one of two consecutive phases.
+        // landed: a warp that rescales waits for it.  The test is exact: P V
+        // (jg + 1) of the same buffer needs this block's P V first.
         if (rescale) {
-          if (!(ok = wait_bar(sh.pv_done, (jg - 1) & 1))) break;
+          if (!(ok = wait_bar(sh.s_free[si ^ 1], ((jg - 1) >> 1) & 1))) break;
           tc_fence_after();
 #pragma unroll 1
           for (int c = 0; c < D / 2; c += 32) {
@@ -872,9 +860,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   // ------------------------------------------------------------ teardown --
   // every MMA issued by this CTA has finished before TMEM is released
-  if (warp == 1) {
-    mma_commit(bar(sh.mma_done));
-    mbar_wait(bar(sh.mma_done), 0);
+  if (warp == 1 || warp == kPvWarp) {
+    uint64_t &done = sh.mma_done[warp == 1 ? 0 : 1];
+    mma_commit(bar(done));
+    mbar_wait(bar(done), 0);
   }
   tc_fence_before();
   __syncthreads();
