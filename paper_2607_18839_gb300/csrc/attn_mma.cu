@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kThreads) attn_stage_kernel(const AttnParams p
     if (d < 0) return;  // grid is an upper bound of the tile count
     const int lt = s_info[1], b0 = s_info[2], b1 = s_info[3];
     bool bad;
-    page_prefix(p, d, pc0, P_d, bad);
+    page_prefix(p, p.prefix_cu, d, pc0, P_d, bad);
     if (bad) flag_error(p.err, HPD_DEVERR_PREFIX_CU);
     doc = d;
     const int R_d = (b1 - b0) * m * G;

@@ -95,6 +95,7 @@ constexpr int kThreads = 32 * (kPvWarp + 1);
 // consumers of a metadata slot: two producers, two MMA issuers, softmax warps
 constexpr uint32_t kMetaConsumers = 4 + kSoftmaxWarps;
 constexpr int kMaxRing = 3;  // largest K / V ring
+constexpr int kStageInts = 2800;  // offsets and lengths staged in shared memory
 
 // Metadata of one unit, written by the scheduler warp.
 struct UnitMeta {
@@ -128,7 +129,8 @@ struct TcLayout {
   static constexpr uint32_t kK = 0;
   static constexpr uint32_t kV = kK + kKStages * kTileBytes;
   static constexpr uint32_t kMeta = kV + kVStages * kTileBytes;  // 2 UnitMeta slots
-  static constexpr uint32_t kBytes = kMeta + 2 * sizeof(UnitMeta);
+  static constexpr uint32_t kStage = kMeta + 2 * sizeof(UnitMeta);
+  static constexpr uint32_t kBytes = kStage + kStageInts * sizeof(int);
   static constexpr uint32_t kDynSmem = kBytes + 1024;   // slack to align to 1024
   // TMEM columns: S of block buffer i at col_s(i), O at kColO, the Q rows of
   // unit slot u at col_q(u) (D / 2 columns: two bf16 per column)
@@ -138,7 +140,8 @@ struct TcLayout {
 };
 
 struct __align__(8) TcShared {
-  uint64_t meta_full[2], meta_empty[2];
+  uint64_t stage_full;
+  uint64_t meta_full[2], tab_full[2], meta_empty[2];  // tab: the packed page ids
   uint64_t k_full[kMaxRing], v_full[kMaxRing];
   uint64_t k_empty[kMaxRing], v_empty[kMaxRing];
   // per S buffer: scores written; P written; P V done (the buffer is free and
@@ -222,8 +225,14 @@ __global__ void __launch_bounds__(kThreads, 1)
   extern __shared__ uint8_t smem_raw[];
   __shared__ TcShared sh;
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  UnitMeta *meta =
-      reinterpret_cast<UnitMeta *>(smem_raw + (sbase - smem_u32(smem_raw)) + L::kMeta);
+  uint8_t *sgen = smem_raw + (sbase - smem_u32(smem_raw));
+  UnitMeta *meta = reinterpret_cast<UnitMeta *>(sgen + L::kMeta);
+  // The step's offsets and lengths, when they fit: the softmax warps fetch
+  // them all at once while the roles start, instead of the scheduler fetching
+  // them one dependent load after another.
+  int *stage = reinterpret_cast<int *>(sgen + L::kStage);
+  const int n_cu = p.n_docs + 1, n_stage = 2 * n_cu + p.B * (p.branch_prefix_len ? 2 : 1);
+  const bool staged = p.n_docs < kStageInts && p.B < kStageInts && n_stage <= kStageInts;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int G = p.G, m = p.m;
   const int TT = kRows / G;  // tokens per 128-row tile
@@ -248,11 +257,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(bar(sh.meta_full[s]), 1);
+      mbar_init(bar(sh.tab_full[s]), 1);
       mbar_init(bar(sh.meta_empty[s]), kMetaConsumers);
       mbar_init(bar(sh.s_full[s]), 1);
       mbar_init(bar(sh.p_full[s]), kSoftmaxWarps);
       mbar_init(bar(sh.s_free[s]), 1);
     }
+    mbar_init(bar(sh.stage_full), 32 * kSoftmaxWarps);
     mbar_init(bar(sh.o_full), 1);
     mbar_init(bar(sh.o_empty), kSoftmaxWarps);
     mbar_init(bar(sh.mma_done[0]), 1);
@@ -275,6 +286,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ------------------------------------------------------- scheduler --
     // Fills slot k & 1 with the k-th unit of this CTA that has keys; units
     // without any get their output written here and are skipped.
+    const int *const branch_cu = staged ? stage : p.branch_cu;
+    const int *const prefix_cu = staged ? stage + n_cu : p.prefix_cu;
+    const int *const branch_len = staged ? stage + 2 * n_cu : p.branch_len;
+    const int *const fork_len =
+        staged && p.branch_prefix_len ? stage + 2 * n_cu + p.B : p.branch_prefix_len;
+    bool fetched = !staged;
     unsigned redo = 0;  // units to run once more
     auto take_redo = [&] {
       unsigned r = 0;
@@ -310,6 +327,13 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (p.unit_order) u = p.unit_order[u];  // longest units first
         }
         const int u_id = u;
+        if (!fetched) {
+          if (!wait_bar(sh.stage_full, 0)) {
+            if (lane == 0) set_abort(sh, p.err);
+            break;
+          }
+          fetched = true;
+        }
         const int us = p.div_S(u), split = u - us * p.S_p;
         const int tile = p.div_Hkv(us), g = us - tile * p.H_kv;
         // the page owning the tile: page d has ceil(#branches(d) * m / TT) tiles
@@ -319,8 +343,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int dd = d0 + lane;
           int tiles = 0, c0 = 0, c1 = 0;
           if (dd < p.n_docs) {
-            c0 = min(max(p.branch_cu[dd], 0), p.B);
-            c1 = min(max(p.branch_cu[dd + 1], 0), p.B);
+            c0 = min(max(branch_cu[dd], 0), p.B);
+            c1 = min(max(branch_cu[dd + 1], 0), p.B);
             if (c1 < c0) {
               flag_error(p.err, HPD_DEVERR_BRANCH_CU);
               c1 = c0;
@@ -349,7 +373,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (d < 0) continue;
         int pc0, P_d;
         bool bad_prefix;
-        page_prefix(p, d, pc0, P_d, bad_prefix);
+        page_prefix(p, prefix_cu, d, pc0, P_d, bad_prefix);
         if (lane == 0 && bad_prefix) flag_error(p.err, HPD_DEVERR_PREFIX_CU);
         const int tok0 = b0 * m + lt * TT;
         const int ntok = min(TT, (b1 - b0) * m - lt * TT);
@@ -362,15 +386,15 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int bl = c0 + lane;
           int np = 0;
           if (bl < nbc) {
-            int Lb = p.branch_len[b_lo + bl];
+            int Lb = branch_len[b_lo + bl];
             const int cap = p.max_pages * kPage;
             if (Lb < 0 || Lb > cap) {
               flag_error(p.err, HPD_DEVERR_BRANCH_LEN);
               Lb = min(max(Lb, 0), cap);
             }
             int f = P_d;
-            if (p.branch_prefix_len) {
-              f = p.branch_prefix_len[b_lo + bl];
+            if (fork_len) {
+              f = fork_len[b_lo + bl];
               if (f < 0 || f > P_d) {
                 flag_error(p.err, HPD_DEVERR_FORK_LEN);
                 f = min(max(f, 0), P_d);
@@ -394,27 +418,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int P_s = base;
         if (lane == 0) M.page_start[nbc] = P_s;
         __syncwarp();
-        // packed suffix page ids: every lookup in flight, then the valid ones kept
-        const int n_tab = min(P_s, kPageCap);
-#pragma unroll 1
-        for (int gp = lane; gp < n_tab; gp += 32) {
-          int lo = 0, hi = nbc;  // largest bl with page_start[bl] <= gp
-          while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (M.page_start[mid] <= gp) lo = mid; else hi = mid;
-          }
-          cp_async4(smem_u32(&M.page_tab[gp]),
-                    p.page_table + static_cast<size_t>(b_lo + lo) * p.max_pages +
-                        (gp - M.page_start[lo]));
-        }
-        cp_async_commit();
-        cp_async_wait<0>();
-#pragma unroll 1
-        for (int gp = lane; gp < n_tab; gp += 32)
-          if (static_cast<unsigned>(M.page_tab[gp]) >= static_cast<unsigned>(p.num_pages)) {
-            flag_error(p.err, HPD_DEVERR_PAGE_ID);
-            M.page_tab[gp] = 0;
-          }
         const int N = ceil_div_i(kmax, kBlk) + ceil_div_i(P_s, kPagesPerBlock);
         // (a unit has fewer than 2^27 blocks and at most 8 splits)
         const int blk_lo = p.div_S(split * N), blk_hi = p.div_S((split + 1) * N);
@@ -437,6 +440,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           continue;
         }
         if (lane == 0) {
+          M.valid = 1;
           M.g = g;
           M.split = split;
           M.tok0 = tok0;
@@ -452,13 +456,38 @@ __global__ void __launch_bounds__(kThreads, 1)
           M.exact = again || *static_cast<volatile int *>(&sh.exact);
           sh.unit_id[k & 31] = u_id;
         }
+        // published without the page ids, which only suffix blocks need
+        __syncwarp();
+        __threadfence_block();
+        if (lane == 0) mbar_arrive(bar(sh.meta_full[slot]));
+        // packed suffix page ids: every lookup in flight, then the valid ones kept
+        const int n_tab = min(P_s, kPageCap);
+#pragma unroll 1
+        for (int gp = lane; gp < n_tab; gp += 32) {
+          int lo = 0, hi = nbc;  // largest bl with page_start[bl] <= gp
+          while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (M.page_start[mid] <= gp) lo = mid; else hi = mid;
+          }
+          cp_async4(smem_u32(&M.page_tab[gp]),
+                    p.page_table + static_cast<size_t>(b_lo + lo) * p.max_pages +
+                        (gp - M.page_start[lo]));
+        }
+        cp_async_commit();
+        cp_async_wait<0>();
+#pragma unroll 1
+        for (int gp = lane; gp < n_tab; gp += 32)
+          if (static_cast<unsigned>(M.page_tab[gp]) >= static_cast<unsigned>(p.num_pages)) {
+            flag_error(p.err, HPD_DEVERR_PAGE_ID);
+            M.page_tab[gp] = 0;
+          }
         have = true;
         break;
       }
-      if (lane == 0) M.valid = have ? 1 : 0;
+      if (!have && lane == 0) M.valid = 0;
       __syncwarp();
       __threadfence_block();
-      if (lane == 0) mbar_arrive(bar(sh.meta_full[slot]));
+      if (lane == 0) mbar_arrive(have ? bar(sh.tab_full[slot]) : bar(sh.meta_full[slot]));
       if (!have) break;
     }
   } else if (warp == 0 || warp == kVWarp) {
@@ -495,6 +524,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!M.valid) break;
       const int g = M.g, nP = M.nP, pc0 = M.pc0, blk_lo = M.blk_lo, nb = M.n_blocks;
       const int P_s = M.page_start[M.nbc];
+      bool tab = false;  // the packed page ids are complete
       // entry -1 of the K ring: the unit's Q tile, tokens [tok0, tok0 + TT),
       // heads of KV head g
 #pragma unroll 1
@@ -505,6 +535,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         // waiting for the ring slot); pages past the last one any row sees
         // repeat it (finite values, never visible).
         int pg = 0;
+        if (!contiguous && jb >= nP && !tab) {
+          if (!(ok = wait_bar(sh.tab_full[slot], (k >> 1) & 1))) break;
+          tab = true;
+        }
         if (!contiguous && lane < kPagesPerBlock) {
           if (jb < nP) {
             pg = prefix_page(p, M.doc, min(jb * kPagesPerBlock + lane, M.pp_last));
@@ -554,6 +588,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                               b, c * 64, g, 0, pgi);
         }
       }
+      if (ok && !tab) ok = wait_bar(sh.tab_full[slot], (k >> 1) & 1);  // written before reuse
       if (!ok) break;
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(sh.meta_empty[slot]));
@@ -672,6 +707,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Warpgroup half h owns key columns [64 h, 64 h + 64) of every block and
     // output columns [64 h, 64 h + 64).
     const int h = (warp - 2) >> 2;        // column half
+    if (staged) {
+#pragma unroll 1
+      for (int i = tid - 64; i < n_stage; i += 32 * kSoftmaxWarps) {
+        const int *src = i < n_cu              ? p.branch_cu + i
+                         : i < 2 * n_cu        ? p.prefix_cu + (i - n_cu)
+                         : i < 2 * n_cu + p.B  ? p.branch_len + (i - 2 * n_cu)
+                                               : p.branch_prefix_len + (i - 2 * n_cu - p.B);
+        cp_async4(smem_u32(stage + i), src);
+      }
+      cp_async_mbar_arrive(bar(sh.stage_full));
+    }
     const int quad = warp & 3;            // TMEM lane quadrant this warp may access
     const int r_in = quad * 32 + lane;    // row within the tile
     const uint32_t t_lane = tmem + (static_cast<uint32_t>(quad * 32) << 16);

@@ -91,10 +91,11 @@ __device__ __forceinline__ void flag_error(uint32_t *err, uint32_t bit) {
 
 // Prefix of page d: its first token pc0 in the contiguous layout and its
 // length P_d, clamped to the buffers (and, paged, to the table width); bad
-// when prefix_cu is out of range (the caller flags HPD_DEVERR_PREFIX_CU).
-__device__ __forceinline__ void page_prefix(const AttnParams &p, int d, int &pc0, int &P_d,
-                                            bool &bad) {
-  const int a0 = p.prefix_cu[d], a1 = p.prefix_cu[d + 1];
+// when prefix_cu (p.prefix_cu or a copy) is out of range (the caller flags
+// HPD_DEVERR_PREFIX_CU).
+__device__ __forceinline__ void page_prefix(const AttnParams &p, const int *prefix_cu, int d,
+                                            int &pc0, int &P_d, bool &bad) {
+  const int a0 = prefix_cu[d], a1 = prefix_cu[d + 1];
   bad = a0 < 0 || a1 < a0 || a1 > p.prefix_tokens;
   pc0 = min(max(a0, 0), p.prefix_tokens);
   P_d = min(max(a1, pc0), p.prefix_tokens) - pc0;
@@ -134,6 +135,11 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, int sr
 // 4-byte async global->shared copy.
 __device__ __forceinline__ void cp_async4(uint32_t dst, const void *src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
+}
+// Arrive on an mbarrier once this thread's cp.async copies so far have landed
+// (the arrival is one of those the barrier was initialised to expect).
+__device__ __forceinline__ void cp_async_mbar_arrive(uint32_t bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 template <int N>

@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kOrderThreads) unit_order_kernel(AttnParams p,
       const int c1 = max(min(max(p.branch_cu[d + 1], 0), p.B), c0);
       int pc0, P_d;
       bool bad;
-      page_prefix(p, d, pc0, P_d, bad);
+      page_prefix(p, p.prefix_cu, d, pc0, P_d, bad);
       c0s[d] = c0;
       c1s[d] = c1;
       pds[d] = P_d;

@@ -485,3 +485,21 @@ def test_scores_that_leave_the_window_of_their_base(hpd, hq, hkv, D, n):
         torch.cuda.synchronize()
         assert op.errors() == 0
         compare(inp, out.float().cpu().numpy(), lse.cpu().numpy(), ref_out, ref_lse)
+
+
+@pytest.mark.parametrize("n_docs,per_doc,fork", [(1, 1398, True), (1, 1399, True), (930, 1, False),
+                                                 (900, 2, True)])
+def test_lengths_at_the_limit_of_what_a_cta_stages(hpd, n_docs, per_doc, fork):
+    # offsets and lengths are staged in shared memory up to 2,800 numbers (two
+    # offsets per page and one more, one or two lengths per branch): just
+    # below, at and beyond; same bounds as every parity case
+    B = n_docs * per_doc
+    rng = np.random.default_rng(54)
+    P = rng.integers(1, 40, size=n_docs)
+    doc = np.repeat(np.arange(n_docs), per_doc)
+    inp = W.build_inputs(P, [per_doc] * n_docs, rng.integers(0, 35, size=B), 1, 4, 2, 64, seed=55,
+                         branch_prefix_len=rng.integers(0, P[doc] + 1) if fork else None)
+    ref_out, ref_lse = oracle.branch_attn(inp)
+    out, lse, err = run_gpu(hpd, inp)
+    assert err == 0
+    compare(inp, out, lse, ref_out, ref_lse)
