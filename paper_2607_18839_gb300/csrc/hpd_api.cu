@@ -356,7 +356,7 @@ hpd_status hpd_branch_attn_marked(const hpd_branch_attn_args *a, hpd_stream_t st
       if (e == cudaSuccess) e = mark(k++);
     }
     // each kernel after the first overlaps its launch with its predecessor
-    if (e == cudaSuccess) e = hpd::launch_branch_attn_tc(p, pl, pl.lpt, s);
+    if (e == cudaSuccess) e = hpd::launch_branch_attn_tc(p, pl, true, s);
     if (e == cudaSuccess) e = mark(k++);
     if (pl.S_p > 1) {
       if (e == cudaSuccess) e = hpd::launch_merge_splits(p, true, s);
