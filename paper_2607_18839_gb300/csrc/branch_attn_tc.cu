@@ -95,7 +95,7 @@ constexpr int kThreads = 32 * (kPvWarp + 1);
 // consumers of a metadata slot: two producers, two MMA issuers, softmax warps
 constexpr uint32_t kMetaConsumers = 4 + kSoftmaxWarps;
 constexpr int kMaxRing = 3;  // largest K / V ring
-constexpr int kStageInts = 2800;  // offsets and lengths staged in shared memory
+constexpr int kStageInts = 2560;  // offsets and lengths staged in shared memory
 
 // Metadata of one unit, written by the scheduler warp.
 struct UnitMeta {

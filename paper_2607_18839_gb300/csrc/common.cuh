@@ -234,6 +234,8 @@ hpd_status check_call_args(const hpd_branch_attn_args *a);
 // Leading workspace bytes that must be zero before a call (error word and
 // tickets); 0 if the scalars are invalid.
 size_t workspace_zero_bytes(const hpd_branch_attn_args *args);
+// beside: may run while the kernel before it on the stream still does (which
+// has waited for everything before itself, and shares no data with this one).
 cudaError_t launch_accept(const __nv_bfloat16 *logits, const int32_t *drafts, int B, int m, int V,
-                          int32_t *out_tokens, int32_t *accepted_len, cudaStream_t s);
+                          int32_t *out_tokens, int32_t *accepted_len, bool beside, cudaStream_t s);
 }  // namespace hpd

@@ -378,7 +378,7 @@ hpd_status hpd_pmtp_accept(const void *logits, const int32_t *drafts, int B, int
   if (st != HPD_OK) return st;
   const cudaError_t e =
       hpd::launch_accept(static_cast<const __nv_bfloat16 *>(logits), drafts, B, m, V, out_tokens,
-                         accepted_len, reinterpret_cast<cudaStream_t>(stream));
+                         accepted_len, false, reinterpret_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? HPD_OK : cuda_fail(e);
 }
 
@@ -400,16 +400,16 @@ hpd_status hpd_decode_step(const hpd_branch_attn_args *a, const void *logits,
   if (!a->workspace || !aligned(a->workspace, kAlign) || a->workspace_bytes < pl.bytes)
     return HPD_ERR_WORKSPACE;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  auto accept_on = [&](cudaStream_t t) {
+  auto accept_on = [&](cudaStream_t t, bool beside) {
     return hpd::launch_accept(static_cast<const __nv_bfloat16 *>(logits), drafts, a->B, a->m, V,
-                              out_tokens, accepted_len, t);
+                              out_tokens, accepted_len, beside, t);
   };
   int dev = 0;
   const int sms = device_sms(&dev);
   if (!step_concurrent(pl, a, sms)) {
     st = hpd_branch_attn(a, stream);
     if (st != HPD_OK) return st;
-    const cudaError_t e = accept_on(s);
+    const cudaError_t e = accept_on(s, pl.use_tc);
     return e == cudaSuccess ? HPD_OK : cuda_fail(e);
   }
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -427,7 +427,7 @@ hpd_status hpd_decode_step(const hpd_branch_attn_args *a, const void *logits,
   if (!ss.ready) {  // first call inside a capture: in order
     st = hpd_branch_attn(a, stream);
     if (st != HPD_OK) return st;
-    e = accept_on(s);
+    e = accept_on(s, pl.use_tc);
     return e == cudaSuccess ? HPD_OK : cuda_fail(e);
   }
   // fork: the second stream waits for everything enqueued on `stream` so
@@ -437,7 +437,7 @@ hpd_status hpd_decode_step(const hpd_branch_attn_args *a, const void *logits,
   e = cudaStreamWaitEvent(ss.side, ss.fork, 0);
   if (e != cudaSuccess) return cuda_fail(e);
   st = hpd_branch_attn(a, stream);
-  cudaError_t ea = st == HPD_OK ? accept_on(ss.side) : cudaSuccess;
+  cudaError_t ea = st == HPD_OK ? accept_on(ss.side, false) : cudaSuccess;
   // join (also after a failed launch, so that a capture is never left forked)
   e = cudaEventRecord(ss.join, ss.side);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ss.join, 0);

@@ -487,10 +487,10 @@ def test_scores_that_leave_the_window_of_their_base(hpd, hq, hkv, D, n):
         compare(inp, out.float().cpu().numpy(), lse.cpu().numpy(), ref_out, ref_lse)
 
 
-@pytest.mark.parametrize("n_docs,per_doc,fork", [(1, 1398, True), (1, 1399, True), (930, 1, False),
+@pytest.mark.parametrize("n_docs,per_doc,fork", [(1, 1278, True), (1, 1279, True), (852, 1, False),
                                                  (900, 2, True)])
 def test_lengths_at_the_limit_of_what_a_cta_stages(hpd, n_docs, per_doc, fork):
-    # offsets and lengths are staged in shared memory up to 2,800 numbers (two
+    # offsets and lengths are staged in shared memory up to 2,560 numbers (two
     # offsets per page and one more, one or two lengths per branch): just
     # below, at and beyond; same bounds as every parity case
     B = n_docs * per_doc
