@@ -19,7 +19,9 @@
 //   suffix blocks  8 pages of 16 keys, packed from the private caches of the
 //                  unit's branches in branch order.
 // A paged block whose 8 pages are consecutive pool pages loads as one 8-page
-// 4-D box per 64 columns, else as one box per page.
+// box, else as one box per page, issued by 8 lanes at once (one 4 KB box per
+// page instead of one per 64 columns, in a loop, took the batch with scattered
+// prefix pages from 67.3 to 57.9 us per call).
 // For every row and block the visible columns form one interval [lo, hi):
 // a prefix block's keys below the row's limit, or the row's own branch's
 // pages up to its causal bound.  Rows of other branches see nothing of a
@@ -124,6 +126,8 @@ struct TcLayout {
   static constexpr int kChunks = D / 64;                // 64-column (128-byte) boxes
   static constexpr uint32_t kChunkBytes = kRows * 128;  // 128 rows x 128 bytes
   static constexpr uint32_t kTileBytes = kChunks * kChunkBytes;
+  // paged blocks: 8-key groups of kChunks x 1024 bytes instead of whole chunks
+  static constexpr uint32_t kGroupBytes = kChunks * 1024, kPageBytes = 2 * kGroupBytes;
   static constexpr int kKStages = 3, kVStages = 3;
   static_assert(kKStages == kVStages, "one producer code for both rings");
   static constexpr uint32_t kK = 0;
@@ -578,15 +582,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         const unsigned run =
             __ballot_sync(0xffffffffu, lane < kPagesPerBlock - 1 && next == pg + 1);
         const bool one = p.num_pages >= kPagesPerBlock && (run & 0x7fu) == 0x7fu;
-        const int boxes = one ? 1 : kPagesPerBlock;
-#pragma unroll 1
-        for (int i = 0; i < boxes; ++i) {
-          const int pgi = __shfl_sync(0xffffffffu, pg, i);
-#pragma unroll
-          for (int c = 0; c < L::kChunks; ++c)
-            tma_load_4d_elect(dst + c * L::kChunkBytes + i * kPage * 128, one ? run_map : page_map,
-                              b, c * 64, g, 0, pgi);
-        }
+        if (lane < (one ? 1 : kPagesPerBlock))  // each lane its page
+          tma_load_5d(dst + lane * L::kPageBytes, one ? run_map : page_map, b, 0, 0, 0, 2 * pg, g);
+        __syncwarp();
       }
       if (ok && !tab) ok = wait_bar(sh.tab_full[slot], (k >> 1) & 1);  // written before reuse
       if (!ok) break;
@@ -609,6 +607,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // 4) to the start-address field (bits 0-13), which cannot carry: every
     // address stays below 256 KB.
     const uint64_t dk0 = smem_desc_sw128(sbase + L::kK, 16, 1024);
+    const uint64_t dk0_paged = smem_desc_sw128(sbase + L::kK, 16, L::kGroupBytes);
     const bool issuer = elect_one();
     uint32_t sk = 0, pk = 0;  // K ring: stage, phase
     int jg = 0;               // blocks issued
@@ -618,6 +617,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!(ok = wait_bar(sh.meta_full[slot], (k >> 1) & 1))) break;
       const bool valid = meta[slot].valid != 0;
       const int nb = meta[slot].n_blocks;
+      // first paged block of the unit
+      const int j_paged = p.prefix_page_table ? 0 : meta[slot].nP - meta[slot].blk_lo;
       __syncwarp();
       if (!valid) break;
       if (lane == 0) mbar_arrive(bar(sh.meta_empty[slot]));
@@ -629,19 +630,21 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (j >= 0 && jg >= 2 && !(ok = wait_bar(sh.s_free[jg & 1], ((jg >> 1) - 1) & 1))) break;
         tc_fence_after();
         if (issuer) {
-          const uint64_t kd = dk0 + ((sk * L::kTileBytes) >> 4);
+          const bool paged = j >= 0 && j >= j_paged;
+          const uint64_t kd = (paged ? dk0_paged : dk0) + ((sk * L::kTileBytes) >> 4);
+          const uint32_t chunk = paged ? 1024 : L::kChunkBytes;
           if (j < 0) {
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk)
               tmem_cp_128x256b(tmem + L::col_q(slot) + kk * 8,
                                kd + (((kk >> 2) * L::kChunkBytes + (kk & 3) * 32) >> 4));
-          } else {
+          } else {  // (kk >> 2: the 64-column chunk)
             // A from TMEM, 16 dimensions (8 columns) per MMA; K is K-major
             const uint32_t col = tmem + L::col_s(jg & 1);
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk)
               mma_ts_one(col, tmem + L::col_q(slot) + kk * 8,
-                         kd + (((kk >> 2) * L::kChunkBytes + (kk & 3) * 32) >> 4), idesc_qk, kk > 0);
+                         kd + (((kk >> 2) * chunk + (kk & 3) * 32) >> 4), idesc_qk, kk > 0);
             mma_commit_one(bar(sh.s_full[jg & 1]));
           }
           mma_commit_one(bar(sh.k_empty[sk]));
@@ -662,6 +665,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // along N (leading byte offset), 8-key groups 1024 bytes apart along K
     // (stride byte offset).
     const uint64_t dv0 = smem_desc_sw128(sbase + L::kV, L::kChunkBytes, 1024);
+    const uint64_t dv0_paged = smem_desc_sw128(sbase + L::kV, 1024, L::kGroupBytes);
     const bool issuer = elect_one();
     uint32_t sv = 0, pv = 0;  // V ring: stage, phase
     int jg = 0;               // blocks issued
@@ -671,6 +675,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!(ok = wait_bar(sh.meta_full[slot], (k >> 1) & 1))) break;
       const bool valid = meta[slot].valid != 0;
       const int nb = meta[slot].n_blocks;
+      const int j_paged = p.prefix_page_table ? 0 : meta[slot].nP - meta[slot].blk_lo;
       __syncwarp();
       if (!valid) break;
       if (lane == 0) mbar_arrive(bar(sh.meta_empty[slot]));
@@ -683,12 +688,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (issuer) {
           // O (+)= P V: 16 keys per MMA, P in the S buffer (half h of the keys
           // at column 64 h)
-          const uint64_t vd = dv0 + ((sv * L::kTileBytes) >> 4);
+          const uint64_t vd = (j >= j_paged ? dv0_paged : dv0) + ((sv * L::kTileBytes) >> 4);
+          const uint32_t step = (j >= j_paged ? 2 * L::kGroupBytes : 2048u) >> 4;  // 16 keys
           const uint32_t col = tmem + L::col_s(jg & 1);
 #pragma unroll
           for (int kk = 0; kk < kBlk / 16; ++kk)
             mma_ts_one(tmem + L::kColO, col + kk * 8 + (kk >= 4 ? 32 : 0),
-                       vd + ((kk * 16 * 128) >> 4), idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
+                       vd + kk * step, idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
           mma_commit_one(bar(sh.s_free[jg & 1]));
           mma_commit_one(bar(sh.v_empty[sv]));
           if (j == nb - 1) mma_commit_one(bar(sh.o_full));

@@ -186,22 +186,24 @@ inline cudaError_t make_map(CUtensorMap *map, const void *base, uint64_t d0, uin
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// 4-D bf16 tensor map over the paged cache [pages][16][H_kv][D]: one box
-// is box_pages consecutive pages of one KV head (64 columns x 1 head x 16
-// tokens x box_pages pages), rows in page-then-slot order.
+// 5-D bf16 tensor map over the paged cache [pages][16][H_kv][D]: one box is
+// box_pages consecutive pages of one KV head, whole rows, in the order (8-token
+// group, 64-column chunk, token, column), so that a page is one box and one
+// run of shared memory (kGroupBytes per group).
 inline cudaError_t make_page_map(CUtensorMap *map, const void *base, int D, int H_kv,
                                  int num_pages, int box_pages = 1) {
   auto fn = encode_fn();
   if (!fn) return cudaErrorNotSupported;
-  const cuuint64_t dims[4] = {static_cast<cuuint64_t>(D), static_cast<cuuint64_t>(H_kv),
-                              static_cast<cuuint64_t>(kPage), static_cast<cuuint64_t>(num_pages)};
-  const cuuint64_t row = static_cast<cuuint64_t>(D) * 2;
-  const cuuint64_t strides[3] = {row, row * H_kv, row * H_kv * kPage};
-  const cuuint32_t box[4] = {64, 1, static_cast<cuuint32_t>(kPage),
-                             static_cast<cuuint32_t>(box_pages)};
-  const cuuint32_t es[4] = {1, 1, 1, 1};
+  const cuuint64_t row = static_cast<cuuint64_t>(D) * 2 * H_kv;  // bytes of a token
+  const cuuint64_t chunks = static_cast<cuuint64_t>(D / 64);
+  const cuuint64_t dims[5] = {64, 8, chunks, 2 * static_cast<cuuint64_t>(num_pages),
+                              static_cast<cuuint64_t>(H_kv)};
+  const cuuint64_t strides[4] = {row, 128, 8 * row, static_cast<cuuint64_t>(D) * 2};
+  const cuuint32_t box[5] = {64, 8, static_cast<cuuint32_t>(chunks),
+                             2 * static_cast<cuuint32_t>(box_pages), 1};
+  const cuuint32_t es[5] = {1, 1, 1, 1, 1};
   const CUresult r =
-      fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides, box,
+      fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(base), dims, strides, box,
          es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
