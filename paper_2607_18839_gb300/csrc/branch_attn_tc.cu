@@ -780,32 +780,53 @@ __global__ void __launch_bounds__(kThreads, 1)
       // halves come to the same answer when that is, and take that block's
       // maximum together (exact: every block's).
       bool based = false;  // every row of the warp has its base
+      // the scores of half a block are ready; its P is
+      auto await_s = [&](int jg) {
+        if (!wait_bar(sh.s_full[jg & 1], (jg >> 1) & 1)) return false;
+        tc_fence_after();
+        return true;
+      };
+      auto signal_p = [&](int jg) {
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(sh.p_full[jg & 1]));
+      };
       for (int j = 0; j < cur.nb; ++j) {
+        // blocks that every row of the warp sees all of, once the bases are
+        // there: nothing to decide
+        if (based && !cur.exact) {
+          const int j_plain = min(cur.nb, cur.n_plain - cur.blk_lo);
+          for (; j < j_plain; ++j) {
+            const int jg = jbase + j;
+            if (!(ok = await_s(jg))) break;
+            inside &= tc::softmax_half_based(t_lane + L::col_s(jg & 1) + h * 64, true, 0, kBlk, sl2,
+                                             m_run, l_half);
+            signal_p(jg);
+          }
+          if (!ok || j >= cur.nb) break;
+        }
         const int jg = jbase + j;
         const int si = jg & 1;
         const int jb = cur.blk_lo + j;
-        const bool plain = jb < cur.n_plain;
-        int lo = 0, hi = kBlk;
-        bool find_max = cur.exact || !based;
-        if (!plain) {
-          if (jb < cur.nP) {
-            hi = min(cur.lim_p - jb * kBlk, kBlk);
-          } else {
-            const int off = (cur.ps - (jb - cur.nP) * kPagesPerBlock) * kPage;  // column of own key 0
-            lo = max(0, off);
-            hi = min(kBlk, off + cur.last + 1);
-          }
-          if (!cur.exact && !based)
-            find_max = __any_sync(0xffffffffu, cur.valid && m_run == NEG_INF && hi > lo);
+        int lo = 0, hi;
+        if (jb < cur.nP) {
+          hi = min(cur.lim_p - jb * kBlk, kBlk);
+        } else {
+          const int off = (cur.ps - (jb - cur.nP) * kPagesPerBlock) * kPage;  // column of own key 0
+          lo = max(0, off);
+          hi = min(kBlk, off + cur.last + 1);
         }
+        const bool find_max =
+            cur.exact ||
+            (!based && __any_sync(0xffffffffu, cur.valid && m_run == NEG_INF && hi > lo));
         // warp-uniform outcome: the tcgen05.ld / st below are warp-collective
-        if (!(ok = wait_bar(sh.s_full[si], (jg >> 1) & 1))) break;
-        tc_fence_after();
+        if (!(ok = await_s(jg))) break;
         const uint32_t s_addr = t_lane + L::col_s(si) + h * 64;
         bool rescale = false;
         float alpha = 1.f;
         if (!find_max) {
-          inside &= tc::softmax_half_based(s_addr, plain, lo - h * 64, hi - h * 64, sl2, m_run, l_half);
+          inside &= tc::softmax_half_based(s_addr, false, lo - h * 64, hi - h * 64, sl2, m_run, l_half);
         } else {
           const int par = jg & 1;
           bool xok = true;
@@ -836,10 +857,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             tmem_st32(t_lane + o_col + c, o);
           }
         }
-        tmem_st_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(sh.p_full[si]));
+        signal_p(jg);
       }
       if (!ok) break;
       if (__any_sync(0xffffffffu, !inside && cur.valid)) {
