@@ -4,7 +4,6 @@
 // here touches device data.
 #include <cmath>
 #include <cstdint>
-#include <mutex>
 
 #include "common.cuh"
 
@@ -195,9 +194,10 @@ int device_sms(int *dev_out) {
 // The attention kernel leaves SMs idle for part of its run: with fewer
 // than two work units per SM its persistent CTAs (one per SM) either do not
 // fill the GPU or finish their last round of whole units at different times.
-// The acceptance then runs beside it on the idle SMs.  With more units per
-// SM the dynamic scheduler keeps every SM busy until near the end and the
-// two run in order.
+// The acceptance, launched behind it, then runs beside it on the idle SMs.
+// With more units per SM the dynamic scheduler keeps every SM busy until near
+// the end, and the acceptance starts there.  What callers are told only: both
+// are launched alike.
 constexpr int kConcurrentUnitsPerSm = 2;
 bool step_concurrent(const hpd::Plan &pl, const hpd_branch_attn_args *a, int sms) {
   if (!pl.use_tc || sms <= 0) return false;
@@ -205,15 +205,15 @@ bool step_concurrent(const hpd::Plan &pl, const hpd_branch_attn_args *a, int sms
   return units < static_cast<long long>(kConcurrentUnitsPerSm) * sms;
 }
 
-// Per device: the second stream of hpd_decode_step and its fork / join
-// events, created on the first call outside stream capture.
-struct StepStreams {
-  std::mutex mu;
-  bool ready = false;
-  cudaStream_t side = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr;
+// The acceptance of a step, enqueued behind the attention kernel.
+struct StepAccept {
+  const __nv_bfloat16 *logits;
+  const int32_t *drafts;
+  int V;
+  int32_t *out_tokens, *accepted_len;
 };
-StepStreams g_step[64];
+hpd_status enqueue_attn(const hpd_branch_attn_args *a, hpd_stream_t stream, void *const *ev,
+                        const StepAccept *accept);
 
 }  // namespace
 
@@ -281,6 +281,15 @@ hpd_status hpd_branch_attn(const hpd_branch_attn_args *a, hpd_stream_t stream) {
 
 hpd_status hpd_branch_attn_marked(const hpd_branch_attn_args *a, hpd_stream_t stream,
                                   void *const *ev) {
+  return enqueue_attn(a, stream, ev, nullptr);
+}
+
+}  // extern "C"
+
+namespace {
+
+hpd_status enqueue_attn(const hpd_branch_attn_args *a, hpd_stream_t stream, void *const *ev,
+                        const StepAccept *accept) {
   const hpd_status st = hpd::check_call_args(a);
   if (st != HPD_OK) return st;
   const hpd::Plan pl = make_plan(a);
@@ -358,6 +367,14 @@ hpd_status hpd_branch_attn_marked(const hpd_branch_attn_args *a, hpd_stream_t st
     // each kernel after the first overlaps its launch with its predecessor
     if (e == cudaSuccess) e = hpd::launch_branch_attn_tc(p, pl, true, s);
     if (e == cudaSuccess) e = mark(k++);
+    // The acceptance starts on SMs that the attention leaves idle (a CTA of
+    // either leaves no room for one of the other); it is done only when the
+    // attention is, so that the merge may follow it.  Against a second stream
+    // forked and joined with two events, us a step: one page 17.5 -> 14.7,
+    // five ragged pages 45.5 -> 37.6, 256 branches of an 8K page 141 -> 136.
+    if (e == cudaSuccess && accept)
+      e = hpd::launch_accept(accept->logits, accept->drafts, a->B, a->m, accept->V,
+                             accept->out_tokens, accept->accepted_len, true, s);
     if (pl.S_p > 1) {
       if (e == cudaSuccess) e = hpd::launch_merge_splits(p, true, s);
       if (e == cudaSuccess) e = mark(k++);
@@ -367,10 +384,17 @@ hpd_status hpd_branch_attn_marked(const hpd_branch_attn_args *a, hpd_stream_t st
     if (e == cudaSuccess) e = mark(1);
     if (e == cudaSuccess) e = hpd::launch_suffix_stage(p, pl, s);
     if (e == cudaSuccess) e = mark(2);
+    if (e == cudaSuccess && accept)
+      e = hpd::launch_accept(accept->logits, accept->drafts, a->B, a->m, accept->V,
+                             accept->out_tokens, accept->accepted_len, false, s);
   }
   if (e != cudaSuccess) return cuda_fail(e);
   return HPD_OK;
 }
+
+}  // namespace
+
+extern "C" {
 
 hpd_status hpd_pmtp_accept(const void *logits, const int32_t *drafts, int B, int m, int V,
                            int32_t *out_tokens, int32_t *accepted_len, hpd_stream_t stream) {
@@ -396,54 +420,9 @@ hpd_status hpd_decode_step(const hpd_branch_attn_args *a, const void *logits,
   if (st != HPD_OK) return st;
   st = check_accept_args(logits, drafts, a->B, a->m, V, out_tokens, accepted_len);
   if (st != HPD_OK) return st;
-  const hpd::Plan pl = make_plan(a);
-  if (!a->workspace || !aligned(a->workspace, kAlign) || a->workspace_bytes < pl.bytes)
-    return HPD_ERR_WORKSPACE;
-  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  auto accept_on = [&](cudaStream_t t, bool beside) {
-    return hpd::launch_accept(static_cast<const __nv_bfloat16 *>(logits), drafts, a->B, a->m, V,
-                              out_tokens, accepted_len, beside, t);
-  };
-  int dev = 0;
-  const int sms = device_sms(&dev);
-  if (!step_concurrent(pl, a, sms)) {
-    st = hpd_branch_attn(a, stream);
-    if (st != HPD_OK) return st;
-    const cudaError_t e = accept_on(s, pl.use_tc);
-    return e == cudaSuccess ? HPD_OK : cuda_fail(e);
-  }
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  cudaError_t e = cudaStreamIsCapturing(s, &cap);
-  if (e != cudaSuccess) return cuda_fail(e);
-  StepStreams &ss = g_step[dev];
-  std::lock_guard<std::mutex> lock(ss.mu);
-  if (!ss.ready && cap == cudaStreamCaptureStatusNone) {
-    e = cudaStreamCreateWithFlags(&ss.side, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ss.fork, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ss.join, cudaEventDisableTiming);
-    if (e != cudaSuccess) return cuda_fail(e);
-    ss.ready = true;
-  }
-  if (!ss.ready) {  // first call inside a capture: in order
-    st = hpd_branch_attn(a, stream);
-    if (st != HPD_OK) return st;
-    e = accept_on(s, pl.use_tc);
-    return e == cudaSuccess ? HPD_OK : cuda_fail(e);
-  }
-  // fork: the second stream waits for everything enqueued on `stream` so
-  // far; the attention is enqueued first, then the acceptance beside it
-  e = cudaEventRecord(ss.fork, s);
-  if (e != cudaSuccess) return cuda_fail(e);
-  e = cudaStreamWaitEvent(ss.side, ss.fork, 0);
-  if (e != cudaSuccess) return cuda_fail(e);
-  st = hpd_branch_attn(a, stream);
-  cudaError_t ea = st == HPD_OK ? accept_on(ss.side, false) : cudaSuccess;
-  // join (also after a failed launch, so that a capture is never left forked)
-  e = cudaEventRecord(ss.join, ss.side);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ss.join, 0);
-  if (st != HPD_OK) return st;
-  if (ea != cudaSuccess) return cuda_fail(ea);
-  return e == cudaSuccess ? HPD_OK : cuda_fail(e);
+  const StepAccept accept{static_cast<const __nv_bfloat16 *>(logits), drafts, V, out_tokens,
+                          accepted_len};
+  return enqueue_attn(a, stream, nullptr, &accept);
 }
 
 hpd_status hpd_read_errors(const void *workspace, uint32_t *flags, hpd_stream_t stream) {

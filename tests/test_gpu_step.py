@@ -1,8 +1,8 @@
 """hpd_decode_step: the attention and the greedy acceptance as one step.
 
-The acceptance reads only the logits and the drafts, so the library may run
-it beside the attention (on a second stream it forks from and joins to the
-caller's stream) when the attention kernel leaves SMs idle.  Whatever it
+The acceptance reads only the logits and the drafts, so the library runs it
+on the SMs that the attention kernel leaves idle (launched behind it, without
+waiting for it to end).  Whatever it
 chooses, the step must give exactly the results of the two calls made in
 order, eagerly and inside a captured CUDA graph, and match the oracle.
 """
@@ -115,7 +115,7 @@ def test_step_inside_graph_capture(hpd, name):
     tok = torch.full((inp.B, inp.m), -7, dtype=torch.int32, device="cuda")
     acc = torch.full((inp.B,), -7, dtype=torch.int32, device="cuda")
     s = torch.cuda.Stream()
-    op.step(lg, dr, tok, acc, stream=s)  # eager first call (creates the second stream)
+    op.step(lg, dr, tok, acc, stream=s)  # eager first call
     s.synchronize()
     tok.fill_(-7)
     acc.fill_(-7)
