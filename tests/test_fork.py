@@ -105,6 +105,26 @@ def test_gpu_parity(n_docs, per_doc, m, p_fork, layout):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("n_docs,per_doc,m,max_pages", [(3, 2, 1, 1), (2, 4, 16, 32),
+                                                        (5, 605, 5, 33), (11, 294, 64, 65)])
+def test_gpu_rows_of_the_page_table(n_docs, per_doc, m, max_pages):
+    # one warp moves a row: rows of one word, of a warp's width and one more,
+    # and more rows than warps (128 CTAs of 8); all whole numbers, so exact
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    case = _case(np.random.default_rng(7 * max_pages + m), n_docs, per_doc, m, max_pages, 0.1)
+    cap = int(case[4][-1]) * (m + 1) + 1
+    ref, err = F.fork_children(*case[:4], FORK, *case[4:], cap=cap)
+    got, gerr = _gpu(case, cap)
+    assert gerr == err == 0
+    nb = ref["new_B"]
+    assert int(got["new_B"][0]) == nb
+    for k in ("parent", "branch_len", "branch_prefix_len", "page_table"):
+        assert np.array_equal(got[k][:nb], ref[k]), k
+
+
+@pytest.mark.gpu
 def test_gpu_capacity_and_bad_offsets():
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
