@@ -75,6 +75,14 @@ def test_many_branches_two_scan_chunks_d64():
     _run(lengths, m=2, H=2, D=64, pages=9000, max_pages=8, steps=3, seed=12)
 
 
+@pytest.mark.parametrize("n,m", [(304, 8), (305, 8), (160, 64)])
+def test_rows_at_the_copy_grid(n, m):
+    # 304 branches of 8 rows fill the copy's largest grid (1,216 CTAs of 256
+    # vectors) exactly; one more, and many more, take further rounds
+    lengths = np.random.default_rng(3).integers(0, 60, size=n).astype(np.int32)
+    _run(lengths, m=m, H=8, D=128, pages=2000, max_pages=9, steps=2, seed=18)
+
+
 def test_m1_all_accepted():
     _run(np.array([0, 15, 16, 17, 31], np.int32), m=1, H=1, D=64, pages=32, max_pages=4,
          steps=3, seed=13, acc_hi=1)
