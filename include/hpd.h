@@ -147,8 +147,9 @@ hpd_status hpd_workspace_init(void *workspace, size_t workspace_bytes, hpd_strea
 hpd_status hpd_branch_attn(const hpd_branch_attn_args *args, hpd_stream_t stream);
 
 /* Number of kernels one hpd_branch_attn call launches for these scalars
- * (0 if they are invalid).  When H_q / H_kv divides 128 the step runs on
- * tcgen05 tensor cores: one persistent kernel for the shared prefix and the
+ * (0 if they are invalid).  When H_q / H_kv divides 128, or the call has more
+ * than 32 stacked rows (B m H_q / H_kv) and prefixes long enough beside its
+ * private keys, the step runs on tcgen05 tensor cores: one persistent kernel for the shared prefix and the
  * private suffixes, preceded by a one-CTA pass that orders its work units
  * longest first when there are at least two units per SM, and followed by a
  * merge kernel when the keys are split across CTAs.

@@ -1,5 +1,7 @@
 // attn_mma.cu -- the two attention stages of the branch-decode step on
-// warp-level bf16 tensor-core MMA (m16n8k16), producing split partials.
+// warp-level bf16 tensor-core MMA (m16n8k16), producing split partials.  They
+// serve the calls whose head ratio does not divide 128 and whose rows are few
+// or whose private keys dominate; the others run on tcgen05.
 //
 // Shared-prefix stage: for page d and KV head g, the query rows of ALL the
 // page's branches that read KV head g are stacked (row r <-> token

@@ -68,7 +68,12 @@
 // once and keeps its loops (producers, page look-ups), and divides by
 // multiplying: 124 KB of instructions became 64 KB, which took one call of
 // c3's shape from 41.4 to 37.6 us, of a scattered paged batch from 75.8 to
-// 68.3 us, and the attention of c5's shape from 133.3 to 129.7 us.
+// 68.3 us, and the attention of c5's shape from 133.3 to 129.7 us.  (77 KB
+// now, with the softmax loop of its own that fully visible blocks have.)
+// What bounds it: per S buffer the chain softmax, P V, S free, Q K^T, of
+// 1,400-1,575 cycles a block against 1,024 of MMA, and whole units: one call
+// of 152 units of 64 blocks, one for each SM, takes 61.3 us (70.6 with 2,100
+// cycles a block), 256 units of the same length 110.5 us (127.1).
 // All waits are bounded; a timeout sets HPD_DEVERR_TIMEOUT, every role
 // leaves its loop, and the CTA drains its in-flight copies and MMAs, frees
 // its TMEM and exits.  No role waits on a hardware barrier (bar.sync) inside

@@ -24,7 +24,7 @@ struct Plan {
   int tiles_max;   // upper bound of prefix row tiles per KV head
   int wr_s;        // warps along rows in the suffix kernel (1, 2, 4)
   int rt_s;        // suffix row tiles per (branch, KV head)
-  bool use_tc;     // whole step on tcgen05 (G divides 128) or warp MMA stages
+  bool use_tc;     // whole step on tcgen05, or on the warp MMA stages
   bool lpt;        // tcgen05: order the units longest first (more units than SMs)
   size_t off_err;    // uint32 error word
   size_t off_ctr;    // int32 tickets [B][H_kv][rt_s]

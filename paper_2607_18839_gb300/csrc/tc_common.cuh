@@ -1,5 +1,5 @@
 // tc_common.cuh -- pieces of the tcgen05 branch-attention kernel: half of a
-// 128-key block of a row's online softmax, and TMA tensor-map encoding on
+// 128-key block of a row's softmax, and TMA tensor-map encoding on
 // the host.
 #pragma once
 

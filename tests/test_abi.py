@@ -199,7 +199,7 @@ def test_launch_plan_of_the_workloads(lib):
     # a large step (96 pages) orders its work units longest first
     assert [hpd.hpd_branch_attn_kernel_name(_workload_args(big_workload()), k) for k in range(2)] == [
         "unit_order", "branch_attn_tc"]
-    # head ratios that do not divide 128 take the warp-MMA stages
+    # few rows of a head ratio that does not divide 128 take the warp-MMA stages
     g3 = W.build_inputs([200], [3], [4, 0, 33], 3, 6, 2, 128, seed=1)
     a = _workload_args(g3)
     assert [hpd.hpd_branch_attn_kernel_name(a, k) for k in range(2)] == ["prefix_stage",
