@@ -164,7 +164,7 @@ struct __align__(8) TcShared {
   // buffered by block parity) and, at the end of a unit, their partial sums;
   // seq counters publish each value ([half][TMEM lane quadrant])
   float xmax[2][2][kRows];  // [half][block parity][row]
-  float xsum[2][kRows];     // [half][row]
+  float xsum[2][2][kRows];  // [unit parity][half][row]
   int xseq[2][2][4];        // [max | sum][half][quadrant]
   // units (by number in this CTA, modulo 32) whose scores left the window of
   // their base and that run once more, with running maxima
@@ -873,10 +873,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       // ---------------------------------------------------- epilogue --
       // row sum over both halves
-      sh.xsum[h][r_in] = l_half;
+      // (Two buffers in turn: a half may be a unit of one or two blocks, of
+      // which its rows see nothing, ahead of the other, which exchange nothing
+      // and need no P of the other's; not two units, as it awaits the other's
+      // sum of the first.)
+      sh.xsum[k & 1][h][r_in] = l_half;
       publish_seq(&sh.xseq[1][h][quad], k + 1);
       if (!(ok = __all_sync(0xffffffffu, await_seq(&sh.xseq[1][h ^ 1][quad], k + 1, sh)))) break;
-      const float l_run = l_half + sh.xsum[h ^ 1][r_in];
+      const float l_run = l_half + sh.xsum[k & 1][h ^ 1][r_in];
       if (!(ok = wait_bar(sh.o_full, k & 1))) break;
       tc_fence_after();
       const float inv = l_run > 0.f ? 1.f / l_run : 0.f;

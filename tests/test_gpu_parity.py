@@ -503,3 +503,28 @@ def test_lengths_at_the_limit_of_what_a_cta_stages(hpd, n_docs, per_doc, fork):
     out, lse, err = run_gpu(hpd, inp)
     assert err == 0
     compare(inp, out, lse, ref_out, ref_lse)
+
+
+def test_short_units_one_after_another(hpd):
+    # pages of very different sizes with split keys: units of one or two blocks,
+    # of which most warps see nothing, follow one another, so that nothing but
+    # the sums at a unit's end keeps the two halves of a row together; every
+    # call gives the bits of the first
+    rng = np.random.default_rng(833427059)
+    P = rng.integers(105, 4580, size=10)
+    C = rng.integers(3, 84, size=10)
+    L = np.clip(np.round(rng.lognormal(4.5, 0.8, size=int(C.sum()))), 1, 1332).astype(int) + 3
+    doc = np.repeat(np.arange(10), C)
+    inp = W.page_the_prefix(W.build_inputs(P, C, L, 3, 4, 2, 128, seed=56,
+                                           branch_prefix_len=rng.integers(2 * P[doc] // 3, P[doc] + 1)),
+                            seed=57)
+    op = hpd.BranchAttn(hpd.DeviceInputs.from_host(inp))
+    out, lse = op()
+    torch.cuda.synchronize()
+    first = out.clone(), lse.clone()
+    for _ in range(1500):
+        op()
+        op()
+        torch.cuda.synchronize()
+        assert torch.equal(op.out, first[0]) and torch.equal(op.lse, first[1])
+    assert op.errors() == 0
