@@ -56,13 +56,19 @@ hpd_status check_scalars(const hpd_branch_attn_args *a) {
 // faster: a packed suffix block serves the m G rows of a branch only, so
 // where private keys dominate the masked rows cost more than the tensor cores
 // gain.  The rule compares a tile's suffix blocks (at the page table's width)
-// with its prefix blocks.  us per call, warp MMA / tcgen05, branches x prefix
-// / private tokens up to:
-//   m G = 3   64 x 1,024 / 1,024  45 / 108;  16 x 1,024 / 64     24.6 / 16.4
-//   m G = 7   64 x 1,024 / 1,024  52 / 58
-//   m G = 10  16 x 2,000 / 100    33 / 20
-//   m G = 12  256 x 1,024 / 1,024  102 / 68;  64 x 64 / 1,024    40 / 58
-//   m G = 14  32 x 100 / 2,048    52 / 66;  256 x 1,024 / 512    119 / 63
+// with its prefix blocks; the line lies where every private key of the table's
+// width would still be there.  us per call, warp MMA / tcgen05, pages x
+// branches, prefix / private tokens of every branch (2 KV heads; 8 for m G = 5,
+// 10 and 15), and the ratio of blocks:
+//   m G = 3   1 x 64, 1,024 / 48     21 / 20   2.8;   4,096 / 240  35 / 35   2.7
+//             1 x 64, 1,024 / 240    25 / 38   11;    8 x 32       44 / 33   11
+//   m G = 5   1 x 64, 1,024 / 240    45 / 31   6.5;   256 / 240    38 / 42   26
+//   m G = 6   1 x 64, 1,024 / 240    26 / 25   5.5;   1,024 / 1,008  42 / 56  22
+//   m G = 9   2 x 12, 1,024 / 240    26 / 20   3.8;   256 / 240    24 / 25   15
+//   m G = 10  1 x 64, 1,024 / 240    56 / 28   3.2;   2 x 12, 256 / 240  26 / 30  13
+//   m G = 15  2 x 12, 256 / 240      26 / 24   9;     256 / 1,008  46 / 50   36
+// Shorter private keys than the table's width move the line further out (571
+// branches of 8 pages on average at a width of 50, m G = 6: 122 / 40).
 // A call of up to 32 stacked rows keeps the launch plan it reports.
 constexpr int kMmaMaxRows = 32;
 bool tc_ragged(const hpd_branch_attn_args *a, int G, int maxP) {
@@ -71,7 +77,7 @@ bool tc_ragged(const hpd_branch_attn_args *a, int G, int maxP) {
   const int tile_branches = std::min(a->B, ceil_div(kTcTileRows, rows));
   const long long suffix =
       ceil_div(static_cast<long long>(tile_branches) * a->max_pages_per_branch, 8);
-  return suffix <= (rows >= 12 ? 16ll : 1ll) * ceil_div(maxP, 128);
+  return suffix <= (rows >= 12 ? 16ll : rows >= 5 ? 5ll : 2ll) * ceil_div(maxP, 128);
 }
 
 hpd::Plan make_plan(const hpd_branch_attn_args *a) {

@@ -76,7 +76,13 @@ SMALL = {
     "long_suffix_splits": lambda: W.build_inputs([64], [2], [2047, 1500], 4, 32, 8, 128, seed=37,
                                                  max_pages=129),
     "custom_scale": lambda: W.build_inputs([90], [2], [7, 9], 2, 4, 2, 64, seed=38, scale=0.3),
-    # G = 3 and G = 5 do not divide 128: these take the warp-MMA prefix kernel
+    # G = 3 and G = 5 do not divide 128: few rows or long private keys take the
+    # warp-MMA kernels, the others the tcgen05 kernel
+    "g3_long_suffix": lambda: W.build_inputs([50], [3], [2047, 1500, 3], 1, 6, 2, 128, seed=58,
+                                             max_pages=129),
+    "g3_many_long_suffixes": lambda: W.build_inputs([200, 50], [30, 12], [300] * 42, 1, 6, 2, 128,
+                                                    seed=59),
+    "g5_d64_few_rows": lambda: W.build_inputs([129], [2], [600, 5], 2, 10, 2, 64, seed=60),
     "g3_warp_mma_prefix": lambda: W.build_inputs([200, 50], [3, 2], [4, 0, 33, 17, 64], 3, 6, 2,
                                                  128, seed=42, branch_prefix_len=[200, 7, 150, 50, 0]),
     "g5_d64_warp_mma_prefix": lambda: W.build_inputs([129], [4], [1, 2, 3, 100], 2, 10, 2, 64,
