@@ -727,8 +727,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                                                : p.branch_prefix_len + (i - 2 * n_cu - p.B);
         cp_async4(smem_u32(stage + i), src);
       }
-      cp_async_mbar_arrive(bar(sh.stage_full));
     }
+    cp_async_mbar_arrive(bar(sh.stage_full));
     const int quad = warp & 3;            // TMEM lane quadrant this warp may access
     const int r_in = quad * 32 + lane;    // row within the tile
     const uint32_t t_lane = tmem + (static_cast<uint32_t>(quad * 32) << 16);
@@ -935,6 +935,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       jbase += cur.nb;
     }
     if (!ok && lane == 0) set_abort(sh, p.err);
+    // Do not exit while a staged copy or its arrival is in flight: only a
+    // scheduler that gets a unit waits for them.
+    mbar_wait(bar(sh.stage_full), 0);
   }
 
   // ------------------------------------------------------------ teardown --

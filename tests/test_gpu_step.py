@@ -190,3 +190,30 @@ def test_step_acceptance_special_values(hpd, name, V_):
     assert op.errors() == 0
     np.testing.assert_array_equal(tok.cpu().numpy(), ref_tok)
     np.testing.assert_array_equal(acc.cpu().numpy(), ref_acc)
+
+
+@pytest.mark.parametrize("empty,H_kv", [(1, 1), (74, 2), (151, 1), (400, 4)])
+def test_step_of_pages_without_branches(hpd, empty, H_kv):
+    # Pages without branches: most CTAs of the attention find no unit (or no
+    # keys) and end at once, with the copies of the offsets that they began
+    # drained, and the acceptance takes their place; every step gives the bits
+    # of the first, and the oracle's results.
+    inp = W.build_inputs([40] * (empty + 1), [0] * empty + [3], [5, 0, 33], 2, 4 * H_kv, H_kv, 64,
+                         seed=520)
+    logits = W.make_logits(inp.B, inp.m, V, 521)
+    ref_tok, ref_acc = oracle.pmtp_accept(logits, np.zeros((inp.B, inp.m), np.int32))
+    lg, dr = to_dev(hpd, logits, np.zeros((inp.B, inp.m), np.int32))
+    op = hpd.BranchAttn(hpd.DeviceInputs.from_host(inp))
+    tok = torch.empty((inp.B, inp.m), dtype=torch.int32, device="cuda")
+    acc = torch.empty((inp.B,), dtype=torch.int32, device="cuda")
+    op.step(lg, dr, tok, acc)
+    first = results(op, tok, acc)
+    ref_out, ref_lse = oracle.branch_attn(inp)
+    assert np.max(np.abs(op.out.float().cpu().numpy() - ref_out)) <= 1e-2
+    assert np.max(np.abs(first[1] - ref_lse)) <= 1e-3
+    np.testing.assert_array_equal(first[2], ref_tok)
+    np.testing.assert_array_equal(first[3], ref_acc)
+    for _ in range(200):
+        op.step(lg, dr, tok, acc)
+    assert_same(results(op, tok, acc), first)
+    assert op.errors() == 0
