@@ -302,9 +302,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         staged && p.branch_prefix_len ? stage + 2 * n_cu + p.B : p.branch_prefix_len;
     bool fetched = !staged;
     unsigned redo = 0;  // units to run once more
+    // (The softmax warps write the words read here meanwhile: one lane reads
+    // for all, so that the warp never takes two ways at once.)
     auto take_redo = [&] {
       unsigned r = 0;
-      if (lane == 0) r = atomicExch(&sh.redo, 0u);
+      if (lane == 0 && *static_cast<volatile unsigned *>(&sh.redo)) r = atomicExch(&sh.redo, 0u);
       return __shfl_sync(0xffffffffu, r, 0);
     };
     for (int k = 0;; ++k) {
@@ -317,7 +319,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool have = false;
       for (;;) {
         int u = 0;
-        if (!redo && *static_cast<volatile unsigned *>(&sh.redo)) redo = take_redo();
+        if (!redo) redo = take_redo();
         const bool again = redo != 0;
         if (again) {
           u = sh.unit_id[__ffs(redo) - 1];
@@ -325,7 +327,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         } else {
           if (lane == 0) u = atomicAdd(p.unit_ctr, 1);
           u = __shfl_sync(0xffffffffu, u, 0);
-          if (aborted(sh)) break;
+          if (__any_sync(0xffffffffu, aborted(sh))) break;
           if (u >= p.n_units) {
             // none left, once the units still running need no second pass
             if (!__all_sync(0xffffffffu, await_units(kSoftmaxWarps * k, sh))) break;

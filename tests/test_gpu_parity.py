@@ -534,3 +534,27 @@ def test_short_units_one_after_another(hpd):
         torch.cuda.synchronize()
         assert torch.equal(op.out, first[0]) and torch.equal(op.lse, first[1])
     assert op.errors() == 0
+
+
+def test_second_passes_between_units_without_keys(hpd):
+    # Several units to a CTA, alternately of pages without any key (their
+    # outputs are written where units are handed out, by rows that do not fill
+    # a warp's last round) and of pages whose scores leave the window of their
+    # base, so that second passes come in while such units are passed over.
+    # Bounds as where scores leave the window: weights rounded to bf16 (2^-9)
+    # times values of up to 4, and the lse's 1e-3.
+    n = 300
+    P = [0 if d % 2 else 260 for d in range(n)]
+    inp = W.build_inputs(P, [3] * n, [5] * (3 * n), 3, 8, 2, 64, seed=61)
+    inp.branch_len = np.where((np.arange(3 * n) // 3) % 2, 0, inp.branch_len).astype(np.int32)
+    k = W.bf16_bits_to_f32(inp.prefix_k).reshape(n // 2, 260, 2, 64)
+    k[:, 200:] *= 130.0
+    inp.prefix_k = W.f32_to_bf16_bits(k.reshape(-1, 2, 64))
+    ref_out, ref_lse = oracle.branch_attn(inp)
+    assert np.max(ref_lse) > 64.0 * np.log(2.0) and np.isneginf(ref_lse).any()
+    op = hpd.BranchAttn(hpd.DeviceInputs.from_host(inp))
+    for _ in range(20):
+        out, lse = op()
+        torch.cuda.synchronize()
+        compare(inp, out.float().cpu().numpy(), lse.cpu().numpy(), ref_out, ref_lse)
+    assert op.errors() == 0
