@@ -103,6 +103,7 @@ constexpr int kThreads = 32 * (kPvWarp + 1);
 constexpr uint32_t kMetaConsumers = 4 + kSoftmaxWarps;
 constexpr int kMaxRing = 3;  // largest K / V ring
 constexpr int kStageInts = 2560;  // offsets and lengths staged in shared memory
+constexpr uint64_t kBlockLimitNs = 10000;  // of a unit's time: a block takes some 0.7 us
 
 // Metadata of one unit, written by the scheduler warp.
 struct UnitMeta {
@@ -211,16 +212,6 @@ __device__ __forceinline__ bool await_seq(const int *flag, int seq, const TcShar
   return load_seq(flag) >= seq || await_seq_slow(flag, seq, &sh.abort);
 }
 
-// Wait (bounded, mostly asleep) until `n` epilogues of softmax warps are done.
-__device__ __noinline__ bool await_units(int n, const TcShared &sh) {
-  const uint64_t t0 = globaltimer();
-  while (load_seq(&sh.units_done) < n) {
-    if (aborted(sh) || globaltimer() - t0 > kWaitLimitNs) return false;
-    __nanosleep(100);
-  }
-  return true;
-}
-
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
     branch_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k,
@@ -302,6 +293,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         staged && p.branch_prefix_len ? stage + 2 * n_cu + p.B : p.branch_prefix_len;
     bool fetched = !staged;
     unsigned redo = 0;  // units to run once more
+    int nb_last = 0, nb_before = 0;  // blocks of the last two units
     // (The softmax warps write the words read here meanwhile: one lane reads
     // for all, so that the warp never takes two ways at once.)
     auto take_redo = [&] {
@@ -329,8 +321,14 @@ __global__ void __launch_bounds__(kThreads, 1)
           u = __shfl_sync(0xffffffffu, u, 0);
           if (__any_sync(0xffffffffu, aborted(sh))) break;
           if (u >= p.n_units) {
-            // none left, once the units still running need no second pass
-            if (!__all_sync(0xffffffffu, await_units(kSoftmaxWarps * k, sh))) break;
+            // none left, once the units still running (the last two) need no
+            // second pass; who gives up here has set the abort word and the error
+            const uint64_t limit =
+                kWaitLimitNs + (static_cast<uint64_t>(nb_last) + nb_before) * kBlockLimitNs;
+            if (!__all_sync(0xffffffffu,
+                            await_count(smem_u32(&sh.units_done), kSoftmaxWarps * k, &sh.abort,
+                                        p.err, HPD_DEVERR_TIMEOUT, limit)))
+              break;
             redo = take_redo();
             if (!redo) break;
             continue;
@@ -467,6 +465,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           M.exact = again || *static_cast<volatile int *>(&sh.exact);
           sh.unit_id[k & 31] = u_id;
         }
+        nb_before = nb_last;
+        nb_last = blk_hi - blk_lo;
         // published without the page ids, which only suffix blocks need
         __syncwarp();
         __threadfence_block();

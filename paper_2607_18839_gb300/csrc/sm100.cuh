@@ -76,6 +76,27 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity,
   return mbar_try_wait(bar, parity) || mbar_wait_slow(bar, parity, abort, limit_ns);
 }
 
+// Wait, mostly asleep, until the count in shared memory that others add to
+// (ordered before by a fence) has reached n.  After limit_ns it gives up and
+// says so: the abort word is set, and `bit` of *err.  False then, or when
+// *abort is set meanwhile.
+static __device__ __noinline__ bool await_count(uint32_t count, int n, int *abort, uint32_t *err,
+                                                uint32_t bit, uint64_t limit_ns) {
+  const uint64_t t0 = globaltimer();
+  for (;;) {
+    int v;
+    asm volatile("ld.acquire.cta.shared::cta.b32 %0, [%1];" : "=r"(v) : "r"(count) : "memory");
+    if (v >= n) return true;
+    if (*reinterpret_cast<volatile int *>(abort)) return false;
+    if (globaltimer() - t0 > limit_ns) {
+      atomicExch(abort, 1);
+      atomicOr(err, bit);
+      return false;
+    }
+    __nanosleep(100);
+  }
+}
+
 // ----------------------------------------------------------------- TMA --
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map, uint32_t bar,
                                             int x, int y, int z, int w, int v) {
