@@ -57,9 +57,9 @@
 //               sees keys of: that maximum is the row's base, and later
 //               blocks take their exponentials against it without waiting
 //               for anything.  Should a score exceed its base by more than
-//               2^64, the unit runs once more with running maxima in every
-//               block (O then rescaled in TMEM when one grows by more than
-//               2^8), and so do the CTA's later units.
+//               2^64, or O come out not finite, the unit runs once more with
+//               running maxima in every block (O then rescaled in TMEM when
+//               one grows by more than 2^8), and so do the CTA's later units.
 // One split: the unit writes the final bf16 output and lse.  Several splits:
 // it writes its normalised fp32 partial and lse for merge.cu.
 // Code size: every CTA fetches the kernel's instructions anew, at some 150
@@ -168,7 +168,8 @@ struct __align__(8) TcShared {
   float xsum[2][2][kRows];  // [unit parity][half][row]
   int xseq[2][2][4];        // [max | sum][half][quadrant]
   // units (by number in this CTA, modulo 32) whose scores left the window of
-  // their base and that run once more, with running maxima
+  // their base, or whose O is not finite, and that run once more, with running
+  // maxima
   unsigned redo;
   int exact;         // set with the first of them: later units run so at once
   int units_done;    // softmax warps that finished a unit's epilogue
@@ -867,12 +868,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         signal_p(jg);
       }
       if (!ok) break;
-      if (__any_sync(0xffffffffu, !inside && cur.valid)) {
-        if (lane == 0) {
-          atomicOr(&sh.redo, 1u << (k & 31));
-          atomicExch(&sh.exact, 1);
-        }
-      }
       // ---------------------------------------------------- epilogue --
       // row sum over both halves
       // (Two buffers in turn: a half may be a unit of one or two blocks, of
@@ -889,12 +884,17 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float lse = l_run > 0.f ? (m_run + __log2f(l_run)) * kLn2 : NEG_INF;
       const bool final_out = p.S_p == 1;
       const size_t slot_pair = static_cast<size_t>(cur.split) * p.rows_total * p.H_q + cur.pair;
+      float2 finite = make_float2(0.f, 0.f);  // NaN once an infinity or NaN is added
 #pragma unroll 1
       for (int c = 0; c < D / 2; c += 32) {
         uint32_t o[32];
         tmem_ld32(t_lane + o_col + c, o);
         tmem_ld_wait32(o);
         if (!cur.valid) continue;
+#pragma unroll
+        for (int e = 0; e < 32; e += 2)
+          finite = __ffma2_rn(make_float2(__uint_as_float(o[e]), __uint_as_float(o[e + 1])),
+                              make_float2(0.f, 0.f), finite);
         const int dc = h * (D / 2) + c;  // output column
         // 32-byte stores: each fills a whole sector of its row
         if (final_out) {
@@ -926,11 +926,20 @@ __global__ void __launch_bounds__(kThreads, 1)
           p.l_part[slot_pair] = lse;
         }
       }
+      // Scores out of the window, or an O that may have overflowed (weights of
+      // up to 2^64 times values beyond 2^63): the unit runs once more.
+      const bool again =
+          !cur.exact && cur.valid && (!inside || !(finite.x == 0.f && finite.y == 0.f));
+      const bool redo = __any_sync(0xffffffffu, again);
       // O may be overwritten by the next unit once every warp has read it
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
         mbar_arrive(bar(sh.o_empty));
+        if (redo) {
+          atomicOr(&sh.redo, 1u << (k & 31));
+          atomicExch(&sh.exact, 1);
+        }
         __threadfence_block();
         atomicAdd(&sh.units_done, 1);
       }

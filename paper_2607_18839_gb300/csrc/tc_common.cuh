@@ -23,7 +23,11 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
 constexpr int kRows = 128;  // stacked query rows of one tile (MMA M)
 constexpr int kBlk = 128;   // keys per block (MMA N of S = Q K^T)
 constexpr float kRescaleLog2 = 8.0f;  // tolerate a stale row max up to 2^8
-constexpr float kWindowLog2 = 64.0f;  // scores this far above a fixed base stay far from overflow
+// Scores up to this far above a fixed base: their weights, and sums of them,
+// stay far from overflow; O = P V overflows where values beyond 2^63 meet them,
+// which its reader finds (with running maxima, weights up to 2^8 leave room for
+// values up to 2^119).
+constexpr float kWindowLog2 = 64.0f;
 
 // A key the row does not see gets the score -inf: 32 columns, visible from
 // lo to hi; scale: multiply by mul first.
@@ -150,7 +154,7 @@ __device__ __forceinline__ bool softmax_half_based(uint32_t s_addr, bool plain, 
   if (!plain) mask32(v + 32, lo - 32, hi - 32, !raw, sl2);
   exp32<true>(s_addr + 16, v + 32, mul, base, sum4, mx4);
   l_half += sum_of(sum4);
-  // (not >, so that a NaN leaves the window too)
+  // (the maxima pass over NaN, which stays in the sums whatever the base)
   return fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * mul <= base + kWindowLog2;
 }
 

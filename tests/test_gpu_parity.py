@@ -558,3 +558,55 @@ def test_second_passes_between_units_without_keys(hpd):
         torch.cuda.synchronize()
         compare(inp, out.float().cpu().numpy(), lse.cpu().numpy(), ref_out, ref_lse)
     assert op.errors() == 0
+
+
+@pytest.mark.parametrize("hq,hkv,D,n", [(16, 2, 128, 40), (8, 2, 64, 3)])
+def test_large_values_under_rising_scores(hpd, hq, hkv, D, n):
+    # Scores that rise by up to some 2^40 above the first block's, inside the
+    # window of their base, meet values of up to 2^112: sums of weights times
+    # values beyond fp32, although every output is a value's size.  Bounds as
+    # where scores leave the window, for outputs in units of 2^110.
+    inp = W.build_inputs([3000, 257], [n, 5], [(13 * b) % 300 for b in range(n + 5)], 4, hq, hkv, D,
+                         seed=62)
+    k = W.bf16_bits_to_f32(inp.prefix_k)
+    k[2500:3000] *= 25.0
+    k[3000 + 140:] *= 25.0
+    inp.prefix_k = W.f32_to_bf16_bits(k)
+    ref_out, ref_lse = oracle.branch_attn(inp)
+    assert 18.0 < np.max(ref_lse) / np.log(2.0) < 60.0
+    for name in ("prefix_v", "v_cache"):
+        v = W.bf16_bits_to_f32(getattr(inp, name)) * np.float32(2.0 ** 110)
+        setattr(inp, name, W.f32_to_bf16_bits(v))
+    op = hpd.BranchAttn(hpd.DeviceInputs.from_host(inp))
+    out, lse = op()
+    torch.cuda.synchronize()
+    assert op.errors() == 0
+    compare(inp, out.double().cpu().numpy() * 2.0 ** -110, lse.cpu().numpy(), ref_out, ref_lse)
+
+
+def test_infinities_and_nan_among_the_keys(hpd):
+    # A row that sees a NaN, or a score of +inf, has no softmax: NaN.  A score
+    # of -inf is a weight of zero.  Rows of the same tile that see neither (their
+    # fork lies before the key, or it is another branch's) are as without them.
+    n = 6
+    inp = W.build_inputs([400, 130], [n, 2], [(29 * b) % 90 for b in range(n + 2)], 3, 8, 2, 64,
+                         seed=63, branch_prefix_len=[400, 300, 129, 128, 350, 0, 130, 129])
+    pk = W.bf16_bits_to_f32(inp.prefix_k)
+    pk[128, 0, 5] = np.inf     # KV head 0: the sign of q decides
+    pk[320, 1] = np.nan        # KV head 1
+    pk[400 + 129, 0, 7] = -np.inf
+    inp.prefix_k = W.f32_to_bf16_bits(pk)
+    kc = W.bf16_bits_to_f32(inp.k_cache)
+    kc[inp.page_table[5, 0], 2, 0] = np.nan
+    inp.k_cache = W.f32_to_bf16_bits(kc)
+    with np.errstate(invalid="ignore"):
+        ref_out, ref_lse = oracle.branch_attn(inp)
+    nan = np.isnan(ref_out)
+    assert np.array_equal(nan.any(-1), nan.all(-1)) and 0.05 < nan.mean() < 0.6
+    for paged in (False, True):
+        out, lse, err = run_gpu(hpd, W.page_the_prefix(inp, seed=64) if paged else inp)
+        assert err == 0
+        np.testing.assert_array_equal(np.isnan(out), nan)
+        assert np.max(np.abs(out[~nan] - ref_out[~nan])) <= OUT_TOL
+        fin = np.isfinite(ref_lse)
+        assert np.max(np.abs(lse[fin] - ref_lse[fin])) <= LSE_TOL
