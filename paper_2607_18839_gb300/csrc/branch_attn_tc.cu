@@ -59,7 +59,9 @@
 //               for anything.  Should a score exceed its base by more than
 //               2^64, or O come out not finite, the unit runs once more with
 //               running maxima in every block (O then rescaled in TMEM when
-//               one grows by more than 2^8), and so do the CTA's later units.
+//               one grows by more than 2^8).  Which units do so is a matter of
+//               their own scores and values alone, so that a call's bits do
+//               not depend on which CTA took which unit.
 // One split: the unit writes the final bf16 output and lse.  Several splits:
 // it writes its normalised fp32 partial and lse for merge.cu.
 // Code size: every CTA fetches the kernel's instructions anew, at some 150
@@ -171,7 +173,6 @@ struct __align__(8) TcShared {
   // their base, or whose O is not finite, and that run once more, with running
   // maxima
   unsigned redo;
-  int exact;         // set with the first of them: later units run so at once
   int units_done;    // softmax warps that finished a unit's epilogue
   int unit_id[32];   // the last units issued
 };
@@ -248,7 +249,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (tid == 0) {
     sh.abort = 0;
     sh.redo = 0u;
-    sh.exact = 0;
     sh.units_done = 0;
     for (int s = 0; s < kMaxRing; ++s) {
       mbar_init(bar(sh.k_full[s]), 1);
@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           M.pp_last = max(kmax - 1, 0) / kPage;
           M.blk_lo = blk_lo;
           M.n_blocks = blk_hi - blk_lo;
-          M.exact = again || *static_cast<volatile int *>(&sh.exact);
+          M.exact = again;
           sh.unit_id[k & 31] = u_id;
         }
         nb_before = nb_last;
@@ -936,10 +936,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) {
         mbar_arrive(bar(sh.o_empty));
-        if (redo) {
-          atomicOr(&sh.redo, 1u << (k & 31));
-          atomicExch(&sh.exact, 1);
-        }
+        if (redo) atomicOr(&sh.redo, 1u << (k & 31));
         __threadfence_block();
         atomicAdd(&sh.units_done, 1);
       }

@@ -610,3 +610,30 @@ def test_infinities_and_nan_among_the_keys(hpd):
         assert np.max(np.abs(out[~nan] - ref_out[~nan])) <= OUT_TOL
         fin = np.isfinite(ref_lse)
         assert np.max(np.abs(lse[fin] - ref_lse[fin])) <= LSE_TOL
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_second_passes_leave_the_bits_of_other_units(hpd, D):
+    # Units that need a second pass among many that do not, several to a CTA:
+    # whichever CTA takes which unit, every call gives the bits of the first,
+    # and a page without such scores the bits of a call of its own.
+    n = 120
+    inp = W.build_inputs([300] * n, [8] * n, [20] * (8 * n), 4, 16, 4, D, seed=65)
+    k = W.bf16_bits_to_f32(inp.prefix_k).reshape(n, 300, 4, D)
+    k[::5, 200:] *= 130.0
+    k[1::5, 200:] *= 25.0  # scores that rise inside the window: another base, other bits
+    inp.prefix_k = W.f32_to_bf16_bits(k.reshape(-1, 4, D))
+    op = hpd.BranchAttn(hpd.DeviceInputs.from_host(inp))
+    out, lse = op()
+    torch.cuda.synchronize()
+    first = out.clone(), lse.clone()
+    for _ in range(300):
+        op()
+    torch.cuda.synchronize()
+    assert torch.equal(op.out, first[0]) and torch.equal(op.lse, first[1])
+    k[::5] = k[2::5]  # no second passes at all: the other pages as they were
+    inp.prefix_k = W.f32_to_bf16_bits(k.reshape(-1, 4, D))
+    calm, calm_lse = hpd.BranchAttn(hpd.DeviceInputs.from_host(inp))()
+    torch.cuda.synchronize()
+    keep = torch.arange(n, device="cuda").repeat_interleave(32) % 5 != 0
+    assert torch.equal(calm[keep], first[0][keep]) and torch.equal(calm_lse[keep], first[1][keep])
