@@ -23,11 +23,19 @@
 // branch, and branch b's children start at new index branch_cu[d+1] + pre_b.
 // Larger calls take two launches (one CTA scans page by page, then many copy).
 // What bounds it: latency, a chain of dependent loads and barriers over a few
-// hundred KB.  A branch's loads are therefore issued together (its flag, its
-// accepted length and its tokens, whichever of them count), every branch's
-// before the first scan, and a page-table row is a warp's, so that its page is
-// looked up once.  768 branches of 65 pages with 54 children, in a graph with
-// the workspace's clearing before it: 14.4 -> 10.3 us a call.
+// hundred KB.  The flags and accepted lengths of all branches are therefore
+// loaded together, then the tokens emitted by layout branches (all tokens of
+// all branches, whichever of them count, were 0.15 us faster at 768 branches
+// and much slower where there are many), all before the first scan, and a
+// page-table row is a warp's, so that its page is looked up once.  us a call,
+// without the workspace's clearing, in a graph: with each branch's loads one
+// after another and a word of the page table to a thread / all tokens / now:
+//   768 branches, 65 pages, m = 8, one in 24 a layout branch    10.8 /  7.1 /  7.3
+//   4,096 branches, 129 pages, m = 16, one in 64                40.7 / 31.4 / 22.3
+//   11,500 branches, 33 pages, m = 64, one in 115                114 /  388 /   49
+//   11,500 branches, 33 pages, m = 64, all                       287 /  395 /  232
+//   20,000 branches, 33 pages, m = 64, one in 100 (two launches) 189 / 1,315 / 189
+// (with 64 CTAs instead of 128: 7.5, 27.2, 55 and 243 us of the first four)
 #include <algorithm>
 
 #include "common.cuh"
@@ -70,14 +78,28 @@ __device__ __forceinline__ int fork_scan(int x, int *ws, int *total) {
   return r;
 }
 
-__device__ __forceinline__ int n_forks(const hpd_fork_args &a, int b) {
-  // every load is issued without waiting for another
+// Tokens of branch b that may hold a fork: those emitted, of a layout branch.
+__device__ __forceinline__ int n_emitted(const hpd_fork_args &a, int b) {
+  // both loads are issued without waiting for one another
   const int lay = a.is_layout ? a.is_layout[b] : 1, n = a.accepted_len[b];
-  const int e = n < 0 || !lay ? 0 : min(n + 1, a.m);
+  return n < 0 || !lay ? 0 : min(n + 1, a.m);
+}
+// The fork tokens among the first e.
+__device__ __forceinline__ int n_forks(const hpd_fork_args &a, int b, int e) {
   const int32_t *tok = a.out_tokens + static_cast<size_t>(b) * a.m;
   int f = 0;
 #pragma unroll 8
-  for (int i = 0; i < a.m; ++i) f += tok[i] == a.fork_token && i < e;
+  for (int i = 0; i < e; ++i) f += tok[i] == a.fork_token;
+  return f;
+}
+// The same of a branch by itself (in the two-launch path, whose one CTA is
+// slower by 5% with the two above).
+__device__ __forceinline__ int n_forks(const hpd_fork_args &a, int b) {
+  if (a.is_layout && !a.is_layout[b]) return 0;
+  const int n = a.accepted_len[b];
+  const int e = n < 0 ? 0 : min(n + 1, a.m);
+  int f = 0;
+  for (int i = 0; i < e; ++i) f += a.out_tokens[static_cast<size_t>(b) * a.m + i] == a.fork_token;
   return f;
 }
 
@@ -197,7 +219,10 @@ __global__ void __launch_bounds__(kFusedThreads) fork_fused_kernel(hpd_fork_args
     }
     return;
   }
-  for (int b = tid; b < a.B; b += kFusedThreads) pre[b] = n_forks(a, b);
+  // every branch's flag and accepted length first, then the tokens that count
+#pragma unroll 4
+  for (int b = tid; b < a.B; b += kFusedThreads) pre[b] = n_emitted(a, b);
+  for (int b = tid; b < a.B; b += kFusedThreads) pre[b] = n_forks(a, b, pre[b]);
   for (int b0 = 0; b0 < a.B; b0 += kFusedThreads) {
     const int b = b0 + tid;
     const int f = b < a.B ? pre[b] : 0;  // this thread's own write

@@ -125,6 +125,35 @@ def test_gpu_rows_of_the_page_table(n_docs, per_doc, m, max_pages):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("n_docs,per_doc,m,p_fork", [(3, 85, 1, 0.5), (1, 256, 64, 0.3),
+                                                     (1, 257, 64, 0.3), (1500, 7, 64, 0.05),
+                                                     (1, 11997, 7, 0.05), (1, 11998, 64, 0.05)])
+def test_gpu_tokens_of_layout_branches_only(n_docs, per_doc, m, p_fork):
+    # The tokens that count are those emitted by layout branches, whatever the
+    # others hold: as many branches as a CTA has threads (256) and one more or
+    # less, the largest call of one launch and the next; whole numbers, exact.
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    rng = np.random.default_rng(9 * per_doc + m)
+    B = n_docs * per_doc
+    lay = (rng.random(B) < 0.1).astype(np.int32)
+    tok = np.where((lay[:, None] == 0) | (rng.random((B, m)) < p_fork), FORK, 5).astype(np.int32)
+    ints = lambda lo, hi, *n: rng.integers(lo, hi, size=n).astype(np.int32)
+    case = [tok, ints(-1, m + 1, B), lay, ints(0, 3000, B),
+            (np.arange(n_docs + 1) * per_doc).astype(np.int32), ints(0, 3000, B), ints(0, 40, B),
+            ints(0, 5000, B, 3)]
+    cap = int(case[4][-1]) + int((case[0] == FORK)[lay == 1].sum()) + 1
+    ref, err = F.fork_children(*case[:4], FORK, *case[4:], cap=cap)
+    got, gerr = _gpu(case, cap)
+    assert gerr == err == 0
+    nb = ref["new_B"]
+    assert int(got["new_B"][0]) == nb
+    for k in ("parent", "branch_len", "branch_prefix_len", "page_table"):
+        assert np.array_equal(got[k][:nb], ref[k]), k
+
+
+@pytest.mark.gpu
 def test_gpu_capacity_and_bad_offsets():
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
