@@ -27,15 +27,20 @@
 // loaded together, then the tokens emitted by layout branches (all tokens of
 // all branches, whichever of them count, were 0.15 us faster at 768 branches
 // and much slower where there are many), all before the first scan, and a
-// page-table row is a warp's, so that its page is looked up once.  us a call,
-// without the workspace's clearing, in a graph: with each branch's loads one
-// after another and a word of the page table to a thread / all tokens / now:
-//   768 branches, 65 pages, m = 8, one in 24 a layout branch    10.8 /  7.1 /  7.3
-//   4,096 branches, 129 pages, m = 16, one in 64                40.7 / 31.4 / 22.3
+// page-table row, or a piece of one, is a warp's, so that its page is looked up
+// once for many words.  us a call, without the workspace's clearing, in a
+// graph: with each branch's loads one after another and a word of the page
+// table to a thread / all tokens / now:
+//   768 branches, 65 pages, m = 8, one in 24 a layout branch    10.8 /  7.1 /  7.4
+//   4,096 branches, 129 pages, m = 16, one in 64                40.7 / 31.4 / 22.5
 //   11,500 branches, 33 pages, m = 64, one in 115                114 /  388 /   49
 //   11,500 branches, 33 pages, m = 64, all                       287 /  395 /  232
 //   20,000 branches, 33 pages, m = 64, one in 100 (two launches) 189 / 1,315 / 189
-// (with 64 CTAs instead of 128: 7.5, 27.2, 55 and 243 us of the first four)
+// (with 64 CTAs instead of 128: 7.6, 27.2, 55 and 243 us of the first four).
+// Whole rows to warps left few branches with wide tables on one CTA; us a call
+// with a word to a thread / whole rows / pieces:
+//   8 branches of 4,096 pages 5.4 / 26 / 4.0, 2 of 16,384 5.0 / 84 / 3.5,
+//   32 of 1,024 7.6 / 10.1 / 5.3
 #include <algorithm>
 
 #include "common.cuh"
@@ -47,6 +52,7 @@ constexpr int kForkThreads = 1024;
 constexpr int kFusedThreads = 256;
 constexpr int kFusedWarps = kFusedThreads / 32;
 constexpr int kFusedGrid = 128;  // CTAs at most: each counts every branch's children
+constexpr int kMaxSegment = 256; // words of a page-table row that a warp takes at most
 constexpr int kMaxFused = 12000;  // B + n_docs + 2 ints of shared memory (48,000 bytes)
 
 // Block-wide exclusive scan of one value per thread; total to *total.
@@ -194,7 +200,7 @@ __global__ void __launch_bounds__(kForkThreads) fork_kernel(hpd_fork_args a) {
 }
 
 // The whole fork step in one launch (see the top of the file).
-__global__ void __launch_bounds__(kFusedThreads) fork_fused_kernel(hpd_fork_args a) {
+__global__ void __launch_bounds__(kFusedThreads) fork_fused_kernel(hpd_fork_args a, int segment) {
   extern __shared__ int s_dyn[];
   int *pre = s_dyn;                 // [B + 1] children of branches before b
   int *cu = s_dyn + a.B + 1;        // [n_docs + 1] branch_cu
@@ -285,9 +291,15 @@ __global__ void __launch_bounds__(kFusedThreads) fork_fused_kernel(hpd_fork_args
       }
     }
   }
-  // page-table rows, one to a warp: the old branches', then the children's (-1)
-  for (int r = blockIdx.x * kFusedWarps + warp; r < a.B + n_children;
-       r += gridDim.x * kFusedWarps) {
+  // page-table rows, a segment of one to a warp: the old branches', then the
+  // children's (-1)
+  const int segs = (a.max_pages - 1) / segment + 1;
+  const long long n_segs = static_cast<long long>(a.B + n_children) * segs;
+  for (long long i = static_cast<long long>(blockIdx.x) * kFusedWarps + warp; i < n_segs;
+       i += static_cast<long long>(gridDim.x) * kFusedWarps) {
+    const int r = segs == 1 ? static_cast<int>(i) : static_cast<int>(i / segs);
+    const int c0 = segs == 1 ? 0 : static_cast<int>(i % segs) * segment;
+    const int c1 = min(a.max_pages - c0, segment) + c0;
     const int32_t *from = nullptr;
     size_t to;
     if (r < a.B) {
@@ -304,7 +316,8 @@ __global__ void __launch_bounds__(kFusedThreads) fork_fused_kernel(hpd_fork_args
       to = static_cast<size_t>(cu[lo + 1]) + c;  // children of page lo after its old branches
     }
     int32_t *row = a.new_page_table + to * a.max_pages;
-    for (int i = lane; i < a.max_pages; i += 32) row[i] = from ? from[i] : -1;
+#pragma unroll 4
+    for (int j = c0 + lane; j < c1; j += 32) row[j] = from ? from[j] : -1;
   }
 }
 
@@ -349,11 +362,16 @@ extern "C" hpd_status hpd_fork_children(const hpd_fork_args *a, hpd_stream_t str
   if (static_cast<long long>(a->B) + a->n_docs + 2 <= hpd::kMaxFused) {
     // one launch; it may start while the previous kernel on the stream
     // finishes (it waits for it before reading anything)
-    const int grid = std::max(1, std::min((a->B + hpd::kFusedWarps - 1) / hpd::kFusedWarps,
-                                          hpd::kFusedGrid));
+    // rows are cut as short as leaves every warp of the grid no more than one
+    // piece, so that few branches with wide tables use many warps too
+    int segment = 32;
+    auto pieces = [&] { return static_cast<long long>(a->B) * ((a->max_pages - 1) / segment + 1); };
+    while (segment < hpd::kMaxSegment && pieces() > hpd::kFusedGrid * hpd::kFusedWarps) segment *= 2;
+    const int grid = static_cast<int>(std::max<long long>(
+        1, std::min<long long>((pieces() + hpd::kFusedWarps - 1) / hpd::kFusedWarps, hpd::kFusedGrid)));
     const size_t smem = sizeof(int) * (static_cast<size_t>(a->B) + a->n_docs + 2);
     e = hpd::launch_kernel(true, hpd::fork_fused_kernel, dim3(grid), dim3(hpd::kFusedThreads), smem,
-                           s, *a);
+                           s, *a, segment);
   } else {
     hpd::fork_kernel<<<1, hpd::kForkThreads, 0, s>>>(*a);
     if (a->B > 0) {

@@ -154,6 +154,30 @@ def test_gpu_tokens_of_layout_branches_only(n_docs, per_doc, m, p_fork):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("B,max_pages", [(1, 32768), (1, 32769), (3, 4097), (31, 1056), (1023, 33),
+                                         (1024, 257), (1025, 256), (700, 1000)])
+def test_gpu_pieces_of_wide_rows(B, max_pages):
+    # a row is cut into pieces of 32 to 256 words, as few pieces as the largest
+    # grid has warps (1,024) where that is enough: full and nearly empty last
+    # pieces, one piece to a warp and more; whole numbers, so exact
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    rng = np.random.default_rng(B + max_pages)
+    ints = lambda lo, hi, *n: rng.integers(lo, hi, size=n).astype(np.int32)
+    tok = np.where(rng.random((B, 2)) < 0.2, FORK, 5).astype(np.int32)
+    tok[-1, 0] = FORK
+    case = [tok, np.full(B, 1, np.int32), None, ints(0, 3000, B), np.array([0, B // 2, B], np.int32),
+            None, ints(0, 40, B), ints(0, 5000, B, max_pages)]
+    cap = B + int((tok == FORK).sum())
+    ref, err = F.fork_children(*case[:4], FORK, *case[4:], cap=cap)
+    got, gerr = _gpu(case, cap)
+    assert gerr == err == 0 and int(got["new_B"][0]) == ref["new_B"] == cap
+    for k in ("parent", "branch_len", "branch_prefix_len", "page_table"):
+        assert np.array_equal(got[k], ref[k]), k
+
+
+@pytest.mark.gpu
 def test_gpu_capacity_and_bad_offsets():
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
