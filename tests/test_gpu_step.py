@@ -217,3 +217,30 @@ def test_step_of_pages_without_branches(hpd, empty, H_kv):
         op.step(lg, dr, tok, acc)
     assert_same(results(op, tok, acc), first)
     assert op.errors() == 0
+
+
+@pytest.mark.parametrize("vocab", [8192, 8193, 10922, 10923])
+def test_acceptance_behind_an_attention_that_may_still_run(hpd, vocab):
+    # An attention call without split keys, then an acceptance call: launched
+    # while the attention runs up to 8,192 values a row, or 2^22 in all (48
+    # branches x 8 rows: 10,922 values), else when it is done.  Exact.
+    inp = W.build_inputs([300] * 16, [3] * 16, [9] * 48, 8, 16, 16, 64, seed=540)
+    op = hpd.BranchAttn(hpd.DeviceInputs.from_host(inp))
+    assert hpd.hpd_branch_attn_kernel_name(op.args, 1) is None
+    rng = np.random.default_rng(541)
+    vals = rng.integers(-40, 41, size=(48, 8, vocab)).astype(np.float32)  # many ties
+    logits = W.f32_to_bf16_bits(vals)
+    ref_tok, _ = oracle.pmtp_accept(logits, np.zeros((48, 8), np.int32))
+    drafts = W.mix_drafts(ref_tok, vocab, 0.8, seed=542)
+    ref_tok, ref_acc = oracle.pmtp_accept(logits, drafts)
+    lg, dr = to_dev(hpd, logits, drafts)
+    tok = torch.empty((48, 8), dtype=torch.int32, device="cuda")
+    acc = torch.empty((48,), dtype=torch.int32, device="cuda")
+    for _ in range(20):
+        tok.fill_(-7), acc.fill_(-7)
+        op()
+        hpd.hpd_pmtp_accept(lg.data_ptr(), dr.data_ptr(), 48, 8, vocab, tok.data_ptr(),
+                            acc.data_ptr(), hpd._stream_handle(None))
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(tok.cpu().numpy(), ref_tok)
+        np.testing.assert_array_equal(acc.cpu().numpy(), ref_acc)
