@@ -198,8 +198,11 @@ hpd_status hpd_pmtp_accept(const void *logits, const int32_t *drafts, int B, int
  * the attention kernel on `stream` with programmatic dependent launch and
  * starts on the SMs that the attention leaves idle: from the start on a
  * one-page step, whose persistent grid is smaller than the SM count, else as
- * its CTAs run out of work.  The step stays ordered on `stream` (work enqueued
- * on `stream` afterwards waits for both) and can be captured in a CUDA graph.
+ * its CTAs run out of work.  Where keys are split, the merge of the splits is
+ * launched before it or after it, whichever leaves the other room; long logits
+ * rows that would crowd on a few idle SMs run after both.  The step stays
+ * ordered on `stream` (work enqueued on `stream` afterwards waits for both) and
+ * can be captured in a CUDA graph.
  */
 hpd_status hpd_decode_step(const hpd_branch_attn_args *args, const void *logits,
                            const int32_t *drafts, int V, int32_t *out_tokens,
@@ -207,9 +210,9 @@ hpd_status hpd_decode_step(const hpd_branch_attn_args *args, const void *logits,
 
 /* 1 when the attention kernel leaves SMs idle for a good part of its run for
  * these host scalars (fewer than two work units per SM; device pointers are
- * not read), so that hpd_decode_step runs the acceptance concurrently with it,
- * 0 when essentially after it, -1 for invalid scalars or an unavailable
- * device. */
+ * not read), so that in hpd_decode_step the acceptance has room beside it, 0
+ * when it runs essentially after it, -1 for invalid scalars or an unavailable
+ * device.  It decides nothing. */
 int hpd_decode_step_concurrent(const hpd_branch_attn_args *args);
 
 /*

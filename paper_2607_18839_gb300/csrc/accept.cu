@@ -197,6 +197,7 @@ __global__ void __launch_bounds__(kAcceptThreads)
   }
   if (!joined) cluster_wait();
   cluster.sync();  // every row's token is in the leader's shared memory
+  pdl_trigger();   // what waits for this kernel (a merge, the next call) may be launched
   if (rank == 0 && threadIdx.x == 0) {
     int k = 0;
     while (k < m && drafts[static_cast<size_t>(b) * m + k] == s_tok[k]) ++k;

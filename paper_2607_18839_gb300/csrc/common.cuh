@@ -82,6 +82,7 @@ struct AttnParams {
   __nv_bfloat16 *out;   // final output, written by the suffix stage
   bool out_align32;     // out is 32-byte aligned (256-bit stores)
   float *lse;           // final lse (may be null)
+  bool accept_next;     // the kernel behind the merge is the acceptance, beside it
 };
 
 // ------------------------------------------------------- device helpers --
@@ -222,6 +223,7 @@ cudaError_t launch_branch_attn_tc(const AttnParams &p, const Plan &plan, bool ov
                                   cudaStream_t s);
 cudaError_t launch_unit_order(const AttnParams &p, int tiles, int *order, cudaStream_t s);
 size_t unit_order_smem_bytes(int n_docs, int B, int tiles);
+long long merge_splits_ctas(long long rows, int H_q);  // CTAs of the merge
 cudaError_t launch_merge_splits(const AttnParams &p, bool overlap, cudaStream_t s);
 cudaError_t launch_wait_selftest(uint32_t *err, uint64_t limit_ns, cudaStream_t s);
 cudaError_t launch_suffix_stage(const AttnParams &p, const Plan &plan, cudaStream_t s);

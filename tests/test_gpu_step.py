@@ -244,3 +244,40 @@ def test_acceptance_behind_an_attention_that_may_still_run(hpd, vocab):
         torch.cuda.synchronize()
         np.testing.assert_array_equal(tok.cpu().numpy(), ref_tok)
         np.testing.assert_array_equal(acc.cpu().numpy(), ref_acc)
+
+
+@pytest.mark.parametrize("B,m,D,vocab", [(38, 8, 128, 80000), (61, 5, 128, 79999), (61, 5, 128, 80000),
+                                         (2, 1, 128, 152064), (61, 5, 64, 80001)])
+def test_step_where_the_acceptance_goes(hpd, B, m, D, vocab):
+    # one page whose keys are split: the acceptance goes behind the merge (304
+    # and 305 long rows, D = 128), before it (a shorter vocabulary, D = 64) or,
+    # with two rows, beside it; whichever it is, the bits of the two calls,
+    # eagerly and from a graph
+    inp = W.build_inputs([1500], [B], [(7 * b) % 50 for b in range(B)], m, 8, 2, D, seed=530)
+    g = torch.Generator(device="cuda").manual_seed(531)
+    lg = torch.randn((B, m, vocab), generator=g, device="cuda").to(torch.bfloat16)
+    best = lg.float().argmax(2).to(torch.int32)
+    dr = torch.where(torch.rand((B, m), generator=g, device="cuda") < 0.8, best, 0).contiguous()
+    op = hpd.BranchAttn(hpd.DeviceInputs.from_host(inp))
+    assert "merge_splits" in [hpd.hpd_branch_attn_kernel_name(op.args, k) for k in range(3)]
+    op()
+    tok, acc = hpd.pmtp_accept(lg, dr)
+    ref = results(op, tok, acc)
+    top = lg.float().gather(2, tok.long()[:, :, None])[:, :, 0]
+    assert torch.equal(top, lg.float().amax(2))
+    tok, acc = torch.full_like(tok, -7), torch.full_like(acc, -7)
+    op.out.zero_()
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    op.step(lg, dr, tok, acc, stream=s)
+    s.synchronize()
+    assert_same(results(op, tok, acc), ref)
+    tok.fill_(-7), acc.fill_(-7), op.out.zero_()
+    s.wait_stream(torch.cuda.current_stream())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        for _ in range(3):
+            op.step(lg, dr, tok, acc, stream=s)
+    graph.replay()
+    assert_same(results(op, tok, acc), ref)
+    assert op.errors() == 0
