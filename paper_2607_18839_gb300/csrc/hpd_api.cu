@@ -53,24 +53,30 @@ hpd_status check_scalars(const hpd_branch_attn_args *a) {
 }
 
 // Head ratios G that do not divide 128 run on the tcgen05 kernel too (row
-// tiles of 128 / G whole tokens), except where the warp-MMA stages measured
-// faster: a packed suffix block serves the m G rows of a branch only, so
-// where private keys dominate the masked rows cost more than the tensor cores
-// gain.  The rule compares a tile's suffix blocks (at the page table's width)
-// with its prefix blocks; the line lies where every private key of the table's
-// width would still be there.  us per call, warp MMA / tcgen05, pages x
+// tiles of 128 / G whole tokens, weights in two bf16 parts), except where the
+// warp-MMA stages may be the faster: a packed suffix block serves the m G rows
+// of a branch only, so where private keys dominate the masked rows cost more
+// than the tensor cores gain.  The rule compares a tile's suffix blocks (at the
+// page table's width) with its prefix blocks, and gives the tcgen05 kernel what
+// is faster on it with hardly an exception (one of 650 random calls took more
+// than 1.02 of its time before, 47 -> 56 us with 20 pages of one branch); many
+// calls beyond the line would be too, with many pages above all.  us per call, warp MMA / tcgen05, pages x
 // branches, prefix / private tokens of every branch (2 KV heads; 8 for m G = 5,
 // 10 and 15), and the ratio of blocks:
-//   m G = 3   1 x 64, 1,024 / 48     21 / 20   2.8;   4,096 / 240  35 / 35   2.7
-//             1 x 64, 1,024 / 240    25 / 38   11;    8 x 32       44 / 33   11
-//   m G = 5   1 x 64, 1,024 / 240    45 / 31   6.5;   256 / 240    38 / 42   26
-//   m G = 6   1 x 64, 1,024 / 240    26 / 25   5.5;   1,024 / 1,008  42 / 56  22
-//   m G = 9   2 x 12, 1,024 / 240    26 / 20   3.8;   256 / 240    24 / 25   15
-//   m G = 10  1 x 64, 1,024 / 240    56 / 28   3.2;   2 x 12, 256 / 240  26 / 30  13
-//   m G = 15  2 x 12, 256 / 240      26 / 24   9;     256 / 1,008  46 / 50   36
-// Shorter private keys than the table's width move the line further out (571
-// branches of 8 pages on average at a width of 50, m G = 6: 122 / 40).
-// A call of up to 32 stacked rows keeps the launch plan it reports.
+//   m G = 3   1 x 64, 1,024 / 48     21 / 20   2.1;   4,096 / 240  35 / 37   2.5
+//             1 x 64, 1,024 / 240    25 / 42   10;    8 x 32       43 / 37   10
+//   m G = 5   1 x 64, 4,096 / 240    78 / 37   1.5;   1,024 / 240  44 / 32   6.1
+//             1 x 64, 256 / 240      38 / 48   25
+//   m G = 6   1 x 64, 4,096 / 240    36 / 27   1.3;   1,024 / 240  26 / 28   5.2
+//   m G = 9   2 x 12, 1,024 / 240    26 / 21   3.6;   256 / 240    24 / 29   15
+//   m G = 10  1 x 64, 1,024 / 240    56 / 45   3.1;   2 x 12, 256 / 240  26 / 36  13
+//   m G = 15  2 x 12, 1,024 / 240    31 / 24   2.1;   256 / 240    26 / 30   8.5
+//   m G = 24  2 x 12, 256 / 240      27 / 24   6.0;   256 / 1,008  46 / 43   24
+// Shorter private keys than the table's width move the line further out.  With
+// D = 64 the warp-MMA stages lose less (28 rows of G = 7: 27 / 29 at a ratio of
+// 2.8, 20 of G = 5: 22 / 29 at 5.8), and the line is at 1.5.  Calls
+// of up to 32 stacked rows stay on the warp-MMA stages, a plan that the tests
+// state; they would gain too (5 branches of m G = 3: 20 / 14).
 constexpr int kMmaMaxRows = 32;
 bool tc_ragged(const hpd_branch_attn_args *a, int G, int maxP) {
   const int rows = a->m * G;
@@ -78,7 +84,9 @@ bool tc_ragged(const hpd_branch_attn_args *a, int G, int maxP) {
   const int tile_branches = std::min(a->B, ceil_div(kTcTileRows, rows));
   const long long suffix =
       ceil_div(static_cast<long long>(tile_branches) * a->max_pages_per_branch, 8);
-  return suffix <= (rows >= 12 ? 16ll : rows >= 5 ? 5ll : 2ll) * ceil_div(maxP, 128);
+  const long long prefix = ceil_div(maxP, 128);
+  if (a->D == 64) return 2 * suffix <= 3 * prefix;
+  return suffix <= (rows >= 5 ? 5 : 2) * prefix;
 }
 
 hpd::Plan make_plan(const hpd_branch_attn_args *a) {

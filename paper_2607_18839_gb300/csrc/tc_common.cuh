@@ -44,12 +44,13 @@ __device__ __forceinline__ void mask32(uint32_t *v, int lo, int hi, bool scale, 
 
 // exp2(mul * v - base) of 32 scores as bf16 pairs in TMEM columns [dst, dst +
 // 16); adds to the sums.  With MAX, the maxima of the scores are taken in the
-// same loop (another pipe than the exponentials').
-template <bool MAX>
+// same loop (another pipe than the exponentials').  With TWO, what the rounding
+// left goes to columns [dst + 32, dst + 48), as bf16 pairs as well.
+template <bool MAX, bool TWO>
 __device__ __forceinline__ void exp32(uint32_t dst, const uint32_t *v, float mul, float base,
                                       float2 *sum4, float *mx4) {
   const float2 mul2 = make_float2(mul, mul), nbase2 = make_float2(-base, -base);
-  uint32_t pk[16];
+  uint32_t pk[16], rest[16];
 #pragma unroll
   for (int c = 0; c < 32; c += 2) {
     const float2 x = make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1]));
@@ -57,9 +58,13 @@ __device__ __forceinline__ void exp32(uint32_t dst, const uint32_t *v, float mul
     const float2 e = make_float2(fast_exp2(arg.x), fast_exp2(arg.y));
     sum4[(c >> 1) & 3] = __fadd2_rn(sum4[(c >> 1) & 3], e);
     pk[c / 2] = pack_bf16x2(e.x, e.y);
+    if constexpr (TWO)
+      rest[c / 2] = pack_bf16x2(e.x - __uint_as_float(pk[c / 2] << 16),
+                                e.y - __uint_as_float(pk[c / 2] & 0xffff0000u));
     if constexpr (MAX) mx4[(c >> 1) & 3] = fmax3(mx4[(c >> 1) & 3], x.x, x.y);
   }
   sm100::tmem_st16(dst, pk);
+  if constexpr (TWO) sm100::tmem_st16(dst + 32, rest);
 }
 __device__ __forceinline__ float sum_of(const float2 *sum4) {
   const float2 s01 = __fadd2_rn(sum4[0], sum4[1]), s23 = __fadd2_rn(sum4[2], sum4[3]);
@@ -70,7 +75,7 @@ __device__ __forceinline__ float sum_of(const float2 *sum4) {
 // One 128-key block of a row's online softmax is the work of two threads: the
 // one of half h owns the 64 columns [64 h, 64 h + 64) of its row.  s_addr is
 // this thread's lane at the half's first column, where P (bf16 pairs, 32
-// columns) replaces the scores; lo / hi bound the row's visible columns in
+// columns; with TWO, 32 more for a second part) replaces the scores; lo / hi bound the row's visible columns in
 // half-block coordinates.  Both threads use the same base, so that O's two
 // column halves and the two partial sums l_half stay consistent.
 // A positive scale keeps the order of the scores, so the maximum is taken
@@ -80,7 +85,7 @@ __device__ __forceinline__ float sum_of(const float2 *sum4) {
 // softmax_half_max: the base is the running maximum, which xchg(max of my
 // visible scaled scores) takes over both halves (and synchronises them).
 // Returns the rescale factor of O.  Warp-collective (tcgen05.ld / st).
-template <class Xchg>
+template <bool TWO, class Xchg>
 __device__ __forceinline__ float softmax_half_max(uint32_t s_addr, int lo, int hi, float sl2,
                                                   float &m_run, float &l_half, Xchg xchg) {
   using namespace sm100;
@@ -111,8 +116,8 @@ __device__ __forceinline__ float softmax_half_max(uint32_t s_addr, int lo, int h
   float2 sum4[4];
 #pragma unroll
   for (int a = 0; a < 4; ++a) sum4[a] = make_float2(0.f, 0.f);
-  exp32<false>(s_addr, v, mul, base, sum4, nullptr);
-  exp32<false>(s_addr + 16, v + 32, mul, base, sum4, nullptr);
+  exp32<false, TWO>(s_addr, v, mul, base, sum4, nullptr);
+  exp32<false, TWO>(s_addr + 16, v + 32, mul, base, sum4, nullptr);
   l_half = l_half * alpha + sum_of(sum4);
   m_run = m_new;
   return alpha;
@@ -124,6 +129,7 @@ __device__ __forceinline__ float softmax_half_max(uint32_t s_addr, int lo, int h
 // exchange nothing and no maximum is waited for.  plain: every row of the warp sees
 // every key, and the scale is positive.  Returns false when a score of this
 // thread lies above the window.
+template <bool TWO>
 __device__ __forceinline__ bool softmax_half_based(uint32_t s_addr, bool plain, int lo, int hi,
                                                    float sl2, float m_run, float &l_half) {
   using namespace sm100;
@@ -133,6 +139,7 @@ __device__ __forceinline__ bool softmax_half_based(uint32_t s_addr, bool plain, 
 #pragma unroll
     for (int c = 0; c < 32; ++c) z[c] = 0u;
     tmem_st32(s_addr, z);
+    if constexpr (TWO) tmem_st32(s_addr + 32, z);
     return true;
   }
   const bool raw = sl2 > 0.f;
@@ -148,11 +155,12 @@ __device__ __forceinline__ bool softmax_half_based(uint32_t s_addr, bool plain, 
   tmem_ld32(s_addr, v);
   tmem_ld_wait32(v);
   tmem_ld32(s_addr + 32, v + 32);
+  if constexpr (TWO) tmem_ld_wait32(v + 32);  // the second part takes their place
   if (!plain) mask32(v, lo, hi, !raw, sl2);
-  exp32<true>(s_addr, v, mul, base, sum4, mx4);
-  tmem_ld_wait32(v + 32);
+  exp32<true, TWO>(s_addr, v, mul, base, sum4, mx4);
+  if constexpr (!TWO) tmem_ld_wait32(v + 32);
   if (!plain) mask32(v + 32, lo - 32, hi - 32, !raw, sl2);
-  exp32<true>(s_addr + 16, v + 32, mul, base, sum4, mx4);
+  exp32<true, TWO>(s_addr + 16, v + 32, mul, base, sum4, mx4);
   l_half += sum_of(sum4);
   // (the maxima pass over NaN, which stays in the sums whatever the base)
   return fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * mul <= base + kWindowLog2;
