@@ -283,8 +283,8 @@ def step_config(name, world):
         "query_tokens_per_step": cfg["B"] * cfg["m"],
         "step": "hpd_decode_step: hpd_branch_attn (shared prefix + private suffix + merge) and "
                 "hpd_pmtp_accept (acceptance inside the step; it reads only the logits and drafts, "
-                "so it runs beside the attention when the attention has fewer than two work units "
-                "per SM and leaves SMs idle, else after it)",
+                "and is launched behind the attention to run on the SMs that this leaves idle, or "
+                "as its CTAs end)",
         "parallelism": f"dp{world} (independent pages per GPU, no collective)",
     }
 
@@ -638,7 +638,7 @@ def measure_workload(name, args, world, rank, dev, stream, H, headline):
                           "t_roofline_us": t_step_roof * 1e6,
                           "frac": t_step_roof / (ms_step * 1e-3)},
         "kernel_us": {k: v * 1e3 for k, v in kernel_ms.items()},
-        "accept_beside_attention": H.hpd_decode_step_concurrent(argsets[0]) == 1,
+        "attention_leaves_sms_idle": H.hpd_decode_step_concurrent(argsets[0]) == 1,
         "accept": {"us_per_call": acc_us, "bytes": per[ACCEPT]["bytes"],
                    "achieved_gbs": per[ACCEPT]["bytes"] / (acc_us * 1e-6) / 1e9,
                    "frac_of_measured_hbm":
@@ -796,7 +796,7 @@ def run_ours(args, world, rank, local):
             "value": r["value"], "ms_per_step": r["ms_per_step"], "roofline": r["roofline"],
             "attention_only": r["attention_only"], "step_roofline": r["step_roofline"],
             "e2e": r["e2e"], "kernel_us": r["kernel_us"], "cold_l2": r["cold_l2"],
-            "accept_beside_attention": r["accept_beside_attention"],
+            "attention_leaves_sms_idle": r["attention_leaves_sms_idle"],
         }
         del r
         torch.cuda.empty_cache()
@@ -839,7 +839,7 @@ def run_ours(args, world, rank, local):
         "kernel_us": head["kernel_us"],
         "accept": head["accept"],
         "cold_l2": head["cold_l2"],
-        "accept_beside_attention": head["accept_beside_attention"],
+        "attention_leaves_sms_idle": head["attention_leaves_sms_idle"],
         "per_config": per_config,
         "kv_append_rollback": head["kv_append_rollback"],
         "fork_children": head["fork_children"],

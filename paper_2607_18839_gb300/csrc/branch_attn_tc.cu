@@ -518,8 +518,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ------------------------------------------------------- producers --
     // The whole warp runs this loop with warp-uniform values; one elected
     // lane issues each copy.  Warp 0: Q and K; warp kVWarp: V.  The K ring
-    // carries each unit's Q tile ahead of its K blocks: ring entry jbase + k
-    // is unit k's Q, entry jg + k + 1 the K of global block jg.
+    // carries each unit's Q tile ahead of its K blocks, as one more entry.
     const bool is_k = warp == 0;
     if (lane == 0) {
       prefetch_tmap(&tm_q);

@@ -193,7 +193,7 @@ hpd_status check_accept_args(const void *logits, const int32_t *drafts, int B, i
 }
 
 // SM count of the current device (cached per device); 0 when unavailable.
-int device_sms(int *dev_out) {
+int device_sms() {
   static int sms[64] = {0};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
@@ -202,17 +202,14 @@ int device_sms(int *dev_out) {
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
     sms[dev] = n;
   }
-  if (dev_out) *dev_out = dev;
   return sms[dev];
 }
 
 // The attention kernel leaves SMs idle for part of its run: with fewer
 // than two work units per SM its persistent CTAs (one per SM) either do not
 // fill the GPU or finish their last round of whole units at different times.
-// The acceptance, launched behind it, then runs beside it on the idle SMs.
 // With more units per SM the dynamic scheduler keeps every SM busy until near
-// the end, and the acceptance starts there.  What callers are told only: both
-// are launched alike.
+// the end.  For callers to know only; a step's launches do not follow from it.
 constexpr int kConcurrentUnitsPerSm = 2;
 bool step_concurrent(const hpd::Plan &pl, const hpd_branch_attn_args *a, int sms) {
   if (!pl.use_tc || sms <= 0) return false;
@@ -466,7 +463,7 @@ hpd_status hpd_pmtp_accept(const void *logits, const int32_t *drafts, int B, int
 
 int hpd_decode_step_concurrent(const hpd_branch_attn_args *args) {
   if (check_scalars(args) != HPD_OK) return -1;
-  const int sms = device_sms(nullptr);
+  const int sms = device_sms();
   if (sms <= 0) return -1;
   return step_concurrent(make_plan(args), args, sms) ? 1 : 0;
 }
