@@ -199,8 +199,7 @@ hpd_status hpd_pmtp_accept(const void *logits, const int32_t *drafts, int B, int
  * starts on the SMs that the attention leaves idle: from the start on a
  * one-page step, whose persistent grid is smaller than the SM count, else as
  * its CTAs run out of work.  Where keys are split, the merge of the splits is
- * launched before it or after it, whichever leaves the other room; long logits
- * rows that would crowd on a few idle SMs run after both.  The step stays
+ * launched before it where it leaves it room, else after it.  The step stays
  * ordered on `stream` (work enqueued on `stream` afterwards waits for both) and
  * can be captured in a CUDA graph.
  */

@@ -26,16 +26,6 @@ constexpr int kAcceptThreads = 256;
 constexpr int kAcceptUnroll = 8;
 constexpr int kMaxCluster = 8;  // portable cluster size
 constexpr int kMaxRows = 64;
-// Short rows, or few values in all: the CTAs may be launched while the kernel
-// before still runs (and wait for it).  Otherwise they would crowd, four to an
-// SM, on the SMs that it leaves idle or leaves first.  us of an attention call
-// without split keys and an acceptance call behind it, launched early / when it
-// is done, rows x values of a row: 20 x 22,294 15.6 / 16.3, 200 x 5,800
-// 22.5 / 23.1, 204 x 20,552 25.9 / 25.9, 276 x 68,217 44.8 / 37.4, 1,278 x
-// 123,024 104 / 84.6; 10 acceptances one after another, 600 x 1,671 5.7 / 6.2.
-constexpr int kEarlyVocab = 8192;
-constexpr long long kEarlyValues = 4ll << 20;
-
 struct ArgBest {
   float v;
   int i;
@@ -213,6 +203,13 @@ __global__ void __launch_bounds__(kAcceptThreads)
 cudaError_t launch_accept(const __nv_bfloat16 *logits, const int32_t *drafts, int B, int m, int V,
                           int32_t *out_tokens, int32_t *accepted_len, bool beside, cudaStream_t s) {
   if (m > kMaxRows) return cudaErrorInvalidValue;
+  // us with the split that the attention left / with much L1: a step of 32 pages,
+  // 24 branches, m = 8, 32,000 values 173.5 / 153.5, one of 608 rows of 52,225
+  // with split keys 44.6 / 35.4; the attention call of 96 branches, m = 8, and an
+  // acceptance call of 149,418 values behind it 83 / 66 (75.1 one by one).
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t pe = prefer_l1(accept_cluster_kernel, done);
+  if (pe != cudaSuccess) return pe;
   const int cs = m < kMaxCluster ? m : kMaxCluster;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(cs) * static_cast<unsigned>(B), 1, 1);
@@ -227,9 +224,7 @@ cudaError_t launch_accept(const __nv_bfloat16 *logits, const int32_t *drafts, in
   cfg.attrs = attr;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
-  const bool early = beside || V <= kEarlyVocab ||
-                     static_cast<long long>(B) * m * V <= kEarlyValues;
-  cfg.numAttrs = early ? 2 : 1;
+  cfg.numAttrs = 2;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, accept_cluster_kernel, logits, drafts, m, V,
                                            out_tokens, accepted_len, beside);
   if (e != cudaSuccess) return e;

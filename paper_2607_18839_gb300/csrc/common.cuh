@@ -1,6 +1,8 @@
 // common.cuh -- device helpers and the internal plan shared by libhpd's kernels.
 #pragma once
 
+#include <atomic>
+
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -227,6 +229,23 @@ long long merge_splits_ctas(long long rows, int H_q);  // CTAs of the merge
 cudaError_t launch_merge_splits(const AttnParams &p, bool overlap, cudaStream_t s);
 cudaError_t launch_wait_selftest(uint32_t *err, uint64_t limit_ns, cudaStream_t s);
 cudaError_t launch_suffix_stage(const AttnParams &p, const Plan &plan, cudaStream_t s);
+// Small shared memory, much L1 for `kernel` (16 of an SM's 228 KB; once per
+// device, `done` remembers).  The attention's CTAs leave their SMs with nearly all
+// of it shared memory, and an SM keeps its split until it is idle: CTAs of a
+// kernel that is launched while the attention runs, and that states no
+// preference, start there at once, with next to no L1 to load through.  Kernels
+// that wait or run beside one another have to ask for the same split.
+template <class K>
+inline cudaError_t prefer_l1(K *kernel, std::atomic<uint64_t> &done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = 1ull << (dev & 63);
+  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 8);  // percent
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_acq_rel);
+  return e;
+}
 // Remember `e` for hpd_last_cuda_error() and return HPD_ERR_CUDA.
 hpd_status record_cuda_error(cudaError_t e);
 // Every host check of an hpd_branch_attn call except the workspace's:

@@ -218,39 +218,19 @@ bool step_concurrent(const hpd::Plan &pl, const hpd_branch_attn_args *a, int sms
 }
 
 // Where the acceptance of a step with split keys goes: it and the merge both
-// follow the attention, and the stream has one order of launches.
-//   beside the merge  the merge is launched first and lets the acceptance start
-//                     at once, so that neither waits for the other: where the
-//                     merge's waiting CTAs leave room on the idle SMs (two to an
-//                     SM), and so with every short step
-//   before the merge  else; the merge then waits for the acceptance
-//   behind it         where the acceptance would crowd.  With D = 128 its CTAs,
-//                     one to a logits row, run four to an SM on the few SMs that
-//                     the attention leaves idle or leaves first, each at a
-//                     fraction of what an SM alone loads; long rows that find no
-//                     room there do better after both
-// us a step in a graph: acceptance on a second stream / beside the merge / before
-// it / behind it; rows, values of a row, SMs the attention leaves idle at most:
-//      8 x 124,315,  88   13.4 / 12.4 / 14.3 /  -        6 x  88,724, 120   10.3 /  9.5 / 10.6 /  -
-//     98 x 139,309,  61   19.1 / 21.7 / 16.4 /  -       52 x 128,857,  24   26.2 /  -   / 21.3 / 24.1
-//     80 x 143,342,   8   38.3 /  -   / 42.1 / 31.6    150 x  81,624,  32   29.7 /  -   / 31.8 / 27.4
-//    576 x 120,248,   8   62.9 /  -   / 68.0 / 46.8    448 x  62,718,   -   37.6 /  -   / 37.2 / 40.5
-// Of 539 random steps of 1 to 430 branches and 5,000 to 152,000 values a row, 6
-// take more than 1.01 of their time with the second stream, at most 1.08 (608
-// rows of 52,225 values: 41.3 -> 44.6); the mean is 0.82.
-constexpr int kBehindVocab = 80000;
-enum AcceptPlace { kBesideMerge, kBeforeMerge, kBehindMerge };
-AcceptPlace accept_place(const hpd::Plan &pl, const hpd_branch_attn_args *a, int V) {
-  if (pl.S_p <= 1) return kBesideMerge;  // there is none
-  const long long rows = static_cast<long long>(a->B) * a->m;
-  auto idle = [&](int tiles) {
-    return std::max(0ll, kPlanSms - static_cast<long long>(tiles) * a->H_kv * pl.S_p);
-  };
-  if (hpd::merge_splits_ctas(pl.rows_total, a->H_q) <= 2 * idle(pl.tiles_max)) return kBesideMerge;
-  // more than 4.5 rows to an idle SM, at the fewest tiles that so many pages have
-  const int tiles = std::max(pl.tiles_max - a->n_docs, std::min(a->n_docs, a->B));
-  if (a->D == 128 && V >= kBehindVocab && 2 * rows > 9 * idle(tiles)) return kBehindMerge;
-  return kBeforeMerge;
+// follow the attention, and the stream has one order of launches.  Where the
+// merge's waiting CTAs leave room on the SMs that the attention leaves idle (two
+// to an SM), the merge is launched first and lets the acceptance start at once,
+// so that neither waits for the other; so with every short step.  Else the
+// acceptance is, and the merge waits for it.  Of their time with the acceptance
+// on a second stream and the merge beside it, in graphs: 60 random steps of one
+// page, 1 to 40 branches and 50,000 to 152,000 values a row take 0.927 so, and
+// 0.957 with the acceptance always first (up to 1.04); 539 steps of all sizes at
+// most 1.006, 0.82 in the mean.
+bool accept_beside_merge(const hpd::Plan &pl, const hpd_branch_attn_args *a) {
+  if (pl.S_p <= 1) return true;  // there is none
+  const long long units = static_cast<long long>(pl.tiles_max) * a->H_kv * pl.S_p;
+  return hpd::merge_splits_ctas(pl.rows_total, a->H_q) <= 2 * std::max(0ll, kPlanSms - units);
 }
 
 // The acceptance of a step, enqueued behind the attention kernel.
@@ -421,19 +401,18 @@ hpd_status enqueue_attn(const hpd_branch_attn_args *a, hpd_stream_t stream, void
     // second stream forked and joined with two events, us a step: one page
     // 17.5 -> 14.7, five ragged pages 45.5 -> 37.6, 256 branches of an 8K page
     // 141 -> 136.
-    const AcceptPlace place = accept ? accept_place(pl, a, accept->V) : kBesideMerge;
-    auto launch_accept = [&](bool beside) {
+    const bool first = accept && !accept_beside_merge(pl, a);
+    auto launch_accept = [&] {
       return hpd::launch_accept(accept->logits, accept->drafts, a->B, a->m, accept->V,
-                                accept->out_tokens, accept->accepted_len, beside, s);
+                                accept->out_tokens, accept->accepted_len, true, s);
     };
-    if (e == cudaSuccess && accept && place == kBeforeMerge) e = launch_accept(true);
+    if (e == cudaSuccess && first) e = launch_accept();
     if (pl.S_p > 1) {
-      p.accept_next = accept && place == kBesideMerge;
+      p.accept_next = accept && !first;
       if (e == cudaSuccess) e = hpd::launch_merge_splits(p, true, s);
       if (e == cudaSuccess) e = mark(k++);
     }
-    if (e == cudaSuccess && accept && place != kBeforeMerge)
-      e = launch_accept(place == kBesideMerge);
+    if (e == cudaSuccess && accept && !first) e = launch_accept();
   } else {
     if (e == cudaSuccess) e = hpd::launch_prefix_stage(p, pl, s);
     if (e == cudaSuccess) e = mark(1);

@@ -87,6 +87,10 @@ cudaError_t launch_merge_splits(const AttnParams &p, bool overlap, cudaStream_t 
   if (p.S_p > kMaxSplits) return cudaErrorInvalidValue;
   const long long blocks = merge_splits_ctas(p.rows_total, p.H_q);
   if (blocks <= 0) return cudaSuccess;
+  static std::atomic<uint64_t> done64{0}, done128{0};  // as the acceptance beside it
+  const cudaError_t e = p.D == 64 ? prefer_l1(merge_splits_kernel<64>, done64)
+                                  : prefer_l1(merge_splits_kernel<128>, done128);
+  if (e != cudaSuccess) return e;
   const dim3 grid(static_cast<unsigned>(blocks));
   return p.D == 64 ? launch_kernel(overlap, merge_splits_kernel<64>, grid, dim3(256), 0, s, p)
                    : launch_kernel(overlap, merge_splits_kernel<128>, grid, dim3(256), 0, s, p);

@@ -219,29 +219,35 @@ def test_step_of_pages_without_branches(hpd, empty, H_kv):
     assert op.errors() == 0
 
 
-@pytest.mark.parametrize("vocab", [8192, 8193, 10922, 10923])
-def test_acceptance_behind_an_attention_that_may_still_run(hpd, vocab):
-    # An attention call without split keys, then an acceptance call: launched
-    # while the attention runs up to 8,192 values a row, or 2^22 in all (48
-    # branches x 8 rows: 10,922 values), else when it is done.  Exact.
-    inp = W.build_inputs([300] * 16, [3] * 16, [9] * 48, 8, 16, 16, 64, seed=540)
+@pytest.mark.parametrize("docs,heads,vocab", [(2, 16, 9001), (16, 16, 9001), (16, 16, 33000)])
+def test_acceptance_behind_an_attention_that_may_still_run(hpd, docs, heads, vocab):
+    # An attention call without split keys, then an acceptance call, which may
+    # be launched at the start of a small attention grid (48 units), or when the
+    # CTAs of a larger one (320) end; both orders in turn.  Exact.
+    inp = W.build_inputs([100] * docs, [3] * docs, [9] * (3 * docs), 8, heads, heads, 64, seed=540)
+    B = 3 * docs
     op = hpd.BranchAttn(hpd.DeviceInputs.from_host(inp))
     assert hpd.hpd_branch_attn_kernel_name(op.args, 1) is None
     rng = np.random.default_rng(541)
-    vals = rng.integers(-40, 41, size=(48, 8, vocab)).astype(np.float32)  # many ties
+    vals = rng.integers(-40, 41, size=(B, 8, vocab)).astype(np.float32)  # many ties
     logits = W.f32_to_bf16_bits(vals)
-    ref_tok, _ = oracle.pmtp_accept(logits, np.zeros((48, 8), np.int32))
+    ref_tok, _ = oracle.pmtp_accept(logits, np.zeros((B, 8), np.int32))
     drafts = W.mix_drafts(ref_tok, vocab, 0.8, seed=542)
     ref_tok, ref_acc = oracle.pmtp_accept(logits, drafts)
     lg, dr = to_dev(hpd, logits, drafts)
-    tok = torch.empty((48, 8), dtype=torch.int32, device="cuda")
-    acc = torch.empty((48,), dtype=torch.int32, device="cuda")
+    tok = torch.empty((B, 8), dtype=torch.int32, device="cuda")
+    acc = torch.empty((B,), dtype=torch.int32, device="cuda")
+    op()
+    torch.cuda.synchronize()
+    first = op.out.clone()
     for _ in range(20):
-        tok.fill_(-7), acc.fill_(-7)
-        op()
-        hpd.hpd_pmtp_accept(lg.data_ptr(), dr.data_ptr(), 48, 8, vocab, tok.data_ptr(),
-                            acc.data_ptr(), hpd._stream_handle(None))
+        tok.fill_(-7), acc.fill_(-7), op.out.zero_()
+        for _ in range(2):
+            op()
+            hpd.hpd_pmtp_accept(lg.data_ptr(), dr.data_ptr(), B, 8, vocab, tok.data_ptr(),
+                                acc.data_ptr(), hpd._stream_handle(None))
         torch.cuda.synchronize()
+        assert torch.equal(op.out, first)
         np.testing.assert_array_equal(tok.cpu().numpy(), ref_tok)
         np.testing.assert_array_equal(acc.cpu().numpy(), ref_acc)
 
@@ -249,10 +255,9 @@ def test_acceptance_behind_an_attention_that_may_still_run(hpd, vocab):
 @pytest.mark.parametrize("B,m,D,vocab", [(38, 8, 128, 80000), (61, 5, 128, 79999), (61, 5, 128, 80000),
                                          (2, 1, 128, 152064), (61, 5, 64, 80001)])
 def test_step_where_the_acceptance_goes(hpd, B, m, D, vocab):
-    # one page whose keys are split: the acceptance goes behind the merge (304
-    # and 305 long rows, D = 128), before it (a shorter vocabulary, D = 64) or,
-    # with two rows, beside it; whichever it is, the bits of the two calls,
-    # eagerly and from a graph
+    # one page whose keys are split: the acceptance goes before the merge (304
+    # and more rows) or, with two rows, beside it; whichever it is, the bits of
+    # the two calls, eagerly and from a graph
     inp = W.build_inputs([1500], [B], [(7 * b) % 50 for b in range(B)], m, 8, 2, D, seed=530)
     g = torch.Generator(device="cuda").manual_seed(531)
     lg = torch.randn((B, m, vocab), generator=g, device="cuda").to(torch.bfloat16)
