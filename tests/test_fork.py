@@ -108,8 +108,8 @@ def test_gpu_parity(n_docs, per_doc, m, p_fork, layout):
 @pytest.mark.parametrize("n_docs,per_doc,m,max_pages", [(3, 2, 1, 1), (2, 4, 16, 32),
                                                         (5, 605, 5, 33), (11, 294, 64, 65)])
 def test_gpu_rows_of_the_page_table(n_docs, per_doc, m, max_pages):
-    # one warp moves a row: rows of one word, of a warp's width and one more,
-    # and more rows than warps (128 CTAs of 8); all whole numbers, so exact
+    # a warp moves a row or a piece of one: rows of one word, of a warp's width
+    # and one more, and more rows than warps (128 CTAs of 8); whole numbers, exact
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no GPU")
